@@ -879,7 +879,9 @@ int group_graph(lsgg_group* g, double dt, bool stale) {
     const GroupRef grp{g->d_B, (int)g->m.size()};
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = launch_group_step(g->m[0]->B, grp, taps, g->stream, &g->ss);
+    bool keep = false;
+    for (const lsgg_ctx* c : g->m) keep = keep || c->B.keep_field;
+    cudaError_t e = launch_group_step(g->m[0]->B, grp, taps, keep, g->stream, &g->ss);
     cudaError_t e2 = cudaStreamEndCapture(g->stream, &graph);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);

@@ -221,7 +221,7 @@ struct StepBuffers {
     int* tile_list;                 // [n_tiles * kTileCap]
     int ntile[3];
     int n_tiles;
-    int field_grid[2], bin_grid;      // field grid: plain / ID-field and debug variants
+    int field_grid[2], bin_grid;      // field grid: values only / with the top two's grains
 };
 
 // A step group: the StepBuffers of several contexts (one GPU, the pass path,
@@ -307,8 +307,9 @@ cudaError_t configure_group_kernels(int n_sm);
 cudaError_t launch_passes_group(const StepBuffers& B0, const GroupRef& grp, int which, int tier, const Taps& taps,
                                 cudaStream_t s);
 cudaError_t launch_bin_group(const StepBuffers& B0, const GroupRef& grp, cudaStream_t s);
-cudaError_t launch_field_group(const StepBuffers& B0, const GroupRef& grp, cudaStream_t s);
-cudaError_t launch_group_step(const StepBuffers& B0, const GroupRef& grp, const Taps& taps, cudaStream_t s,
+cudaError_t launch_field_group(const StepBuffers& B0, const GroupRef& grp, bool ids, cudaStream_t s);
+// (keep: a member stores the top-two field)
+cudaError_t launch_group_step(const StepBuffers& B0, const GroupRef& grp, const Taps& taps, bool keep, cudaStream_t s,
                               const StepStreams* ss);
 // member k's step limit := lim[k] (device array of grp.n entries)
 cudaError_t launch_group_limits(const GroupRef& grp, const long long* lim, cudaStream_t s);

@@ -722,16 +722,19 @@ k_clear_tiles_group(GroupRef grp) {
 // ---------------------------------------------------------------------------
 // Thread (x, y) of a tile owns the column of kTileZ cells at (x, y); for each
 // box covering the column it loads the box's phi_p there and keeps the two
-// largest (phi_p, grain) pairs per cell in registers, ordered by phi_p and,
-// at equal phi_p, by the smaller grain id first -- the order of the
-// box-streaming kernels' 64-bit keys (phi_p, -id) under atomicMax, so m and
-// the ID-field are identical.  Per listed box the CTA first stages, in shared
+// largest values per cell (where wanted with their grains) in registers,
+// ordered by phi_p and, at equal phi_p, by the smaller grain id first -- the
+// order of the box-streaming kernels' 64-bit keys (phi_p, -id) under
+// atomicMax, so m and the ID-field are identical.  Per listed box the CTA first stages, in shared
 // memory, how the tile maps into the box: on an axis where the box's cells
 // in the tile keep one box-local offset (all but boxes spanning nearly the
 // whole domain), the mask of the tile's rows / columns / planes it covers
 // and one arena offset for the tile's corner, so that the per-thread work is
 // a mask test per column and an add per cell; other boxes take the general
 // cyclic path.
+// CTAs per SM the value-only field pass is sized for.
+constexpr int kFieldBlocks = 5;
+
 struct TileBox {
     long long off;            // affine: arena offset of tile cell (0, 0, 0); general: of the box
     int nx, ny;               // box x, y sides
@@ -795,24 +798,42 @@ __device__ __forceinline__ void stage_tile_box(const StepBuffers& B, int b, int 
     t.zm = m;
 }
 
-// (v, id) enters the top two (v1, i1) >= (v2, i2) of a cell; absent entries
-// are (-inf, -1), and v = -inf never enters.
+// (v, id) enters the top two (v1, i1) >= (v2, i2) of a cell; boxes come in
+// ascending grain id, so an equal value never displaces an earlier one (the
+// lowest id on ties).  Absent entries are (-inf, -1).
 __device__ __forceinline__ void top2_insert(float v, int id, float& v1, int& i1, float& v2, int& i2) {
-    const bool c1 = v > v1 || (v == v1 && id < i1);
-    const bool c2 = v > v2 || (v == v2 && id < i2);
-    v2 = c1 ? v1 : (c2 ? v : v2);
+    const bool c1 = v > v1, c2 = v > v2;
     i2 = c1 ? i1 : (c2 ? id : i2);
-    v1 = c1 ? v : v1;
     i1 = c1 ? id : i1;
+    v2 = fmaxf(v2, fminf(v1, v));
+    v1 = fmaxf(v1, v);
 }
 
-// Four CTAs per SM for the plain field; the ID-field and debug variants keep
-// the registers of three.
-template <bool IDF, bool DBG, bool GRP>
-__global__ void __launch_bounds__(kTileX * kTileY, (IDF || DBG || GRP) ? 3 : 4)
+// The two largest values alone.
+__device__ __forceinline__ void top2_values(float v, float& v1, float& v2) {
+    v2 = fmaxf(v2, fminf(v1, v));
+    v1 = fmaxf(v1, v);
+}
+
+// IDS: the grains of the top two are wanted as well (the ID-field, the
+// intermediates of a debug step, the stored field).  Without them the values
+// suffice: a box cell whose phi_p equals the largest value is either its
+// holder, whose m is the second value, or ties with it, and then the two
+// values are equal; every other cell's m is the largest value.  The insertion
+// is then three instructions a cell instead of twelve and the top two take 16
+// registers instead of 32.  The pass is bound by the latency of its column
+// loads (each warp load touches four rows of eight cells, about two 32-byte
+// sectors a row): the freed registers go into a fifth CTA per SM.  Measured on
+// GB300, 256^3 / 5000 grains, whole step: 2.33 ms with the grains tracked at
+// four CTAs, 2.26 / 2.23 / 2.42 ms values only at four / five / six CTAs (six
+// spills).
+template <bool IDS, bool IDF, bool DBG, bool GRP>
+__global__ void __launch_bounds__(kTileX * kTileY, IDS ? 3 : (GRP ? 4 : kFieldBlocks))
 p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
     static_assert(!(GRP && (IDF || DBG)), "step groups run ideal growth without intermediates");
+    static_assert(IDS || !(IDF || DBG), "the ID-field and the intermediates need the top two's grains");
     __shared__ TileBox s_tb[kTileCap];
+    __shared__ int s_id[IDS ? kTileCap : 1];
     __shared__ int s_gb[GRP ? kMaxGroup + 1 : 1];
     if (!GRP && halted(B1)) return;
     const int n_all = GRP ? group_scan(grp, kItemTiles, 0, true, s_gb) : B1.n_tiles;
@@ -822,6 +843,7 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
         const StepBuffers& B = member<GRP>(B1, grp, s_gb, gtile, tile);
         const Domain D = B.dom;
         const float eps = D.eps;
+        const float* const Y = B.Y;
         const int ntx = B.ntile[0], nty = B.ntile[1];
         const int tx = tile % ntx, tyz = tile / ntx, ty = tyz % nty, tz = tyz / nty;
         const int tx0 = tx * kTileX, ty0 = ty * kTileY, z0 = tz * kTileZ;
@@ -832,24 +854,28 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
         const int cnt = B.tile_cnt[tile];
         const bool all = cnt > kTileCap;            // list overflowed: test every box in batches
         const int n_total = all ? B.n_boxes : cnt;
-        float v1[kTileZ], v2[kTileZ], w1[kTileZ], w2[kTileZ];
-        int i1[kTileZ], i2[kTileZ];
+        float v1[kTileZ], v2[kTileZ];
+        int i1[IDS ? kTileZ : 1], i2[IDS ? kTileZ : 1];
 #pragma unroll
-        for (int zz = 0; zz < kTileZ; ++zz) { v1[zz] = v2[zz] = -INFINITY; i1[zz] = i2[zz] = -1; }
+        for (int zz = 0; zz < kTileZ; ++zz) {
+            v1[zz] = v2[zz] = -INFINITY;
+            if (IDS) i1[zz] = i2[zz] = -1;
+        }
         // two sweeps over the tile's boxes: 0 builds the top two, 1 writes phi_c
 #pragma unroll
         for (int sweep = 0; sweep < 2; ++sweep) {
             if (sweep == 1) {
                 ulonglong2* T2 = reinterpret_cast<ulonglong2*>(B.T);
-                const bool keep = B.keep_field != 0;
+                const bool keep = IDS && B.keep_field != 0;
 #pragma unroll
                 for (int zz = 0; zz < kTileZ; ++zz) {
-                    if (keep && col && zz < nzt)
+                    if (IDS && keep && col && zz < nzt)
                         T2[((long long)(z0 + zz) * D.ny + y) * D.nx + x] =
                             make_ulonglong2(i1[zz] >= 0 ? make_key(v1[zz], i1[zz]) : 0ull,
                                             i2[zz] >= 0 ? make_key(v2[zz], i2[zz]) : 0ull);
-                    w1[zz] = i1[zz] >= 0 ? v1[zz] + 0.0f : -eps;
-                    w2[zz] = i2[zz] >= 0 ? v2[zz] + 0.0f : -eps;
+                    // as m: absent is -eps, -0 becomes +0
+                    v1[zz] = v1[zz] > -INFINITY ? v1[zz] + 0.0f : -eps;
+                    v2[zz] = v2[zz] > -INFINITY ? v2[zz] + 0.0f : -eps;
                 }
             }
             for (int base = 0; base < n_total; base += kTileCap) {
@@ -857,9 +883,21 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
                 // one batch (the tile's whole list): the first sweep's staging serves both
                 if (sweep == 0 || n_total > kTileCap) {
                     __syncthreads();                // previous batch done with s_tb
-                    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-                        const int b = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
-                        stage_tile_box(B, b, tx0, ty0, z0, ext_x, ext_y, nzt, s_tb[k]);
+                    if constexpr (IDS) {            // in ascending id: each box's rank in the list
+                        for (int k = threadIdx.x; k < nb; k += blockDim.x)
+                            s_id[k] = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
+                        __syncthreads();
+                        for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+                            const int b = s_id[k];
+                            int rank = 0;
+                            for (int q = 0; q < nb; ++q) rank += s_id[q] < b;
+                            stage_tile_box(B, b, tx0, ty0, z0, ext_x, ext_y, nzt, s_tb[rank]);
+                        }
+                    } else {
+                        for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+                            const int b = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
+                            stage_tile_box(B, b, tx0, ty0, z0, ext_x, ext_y, nzt, s_tb[k]);
+                        }
                     }
                     __syncthreads();
                 }
@@ -869,57 +907,64 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
                     const unsigned zaff = t.zm;
                     const unsigned zm = zaff & 0xffu;
                     const int id = t.id, ps = t.ps;
-                    long long o[kTileZ];                // arena offsets of the column's cells
+                    // the column's cells at arena offsets oc + lz(zz) * ps
+                    auto cells = [&](const long long oc, auto lz) {
+                        const float* yc = Y + oc;
+                        float v[kTileZ];
+                        if (zm == 0xffu) {              // the whole column (uniform)
+#pragma unroll
+                            for (int zz = 0; zz < kTileZ; ++zz) v[zz] = __ldg(yc + (size_t)(lz(zz) * (unsigned)ps));
+                        } else {
+#pragma unroll
+                            for (int zz = 0; zz < kTileZ; ++zz)
+                                v[zz] = (zm >> zz) & 1u ? __ldg(yc + (size_t)(lz(zz) * (unsigned)ps)) : -INFINITY;
+                        }
+                        if (sweep == 0) {
+#pragma unroll
+                            for (int zz = 0; zz < kTileZ; ++zz) {
+                                if constexpr (IDS) top2_insert(v[zz], id, v1[zz], i1[zz], v2[zz], i2[zz]);
+                                else top2_values(v[zz], v1[zz], v2[zz]);
+                            }
+                        } else {
+                            float* zc = B.Z + oc;
+#pragma unroll
+                            for (int zz = 0; zz < kTileZ; ++zz) {
+                                if (!((zm >> zz) & 1u)) continue;
+                                const size_t o = lz(zz) * (unsigned)ps;
+                                bool top;
+                                if constexpr (IDS) top = i1[zz] == id;
+                                else top = v[zz] == v1[zz];
+                                const float m = top ? v2[zz] : v1[zz];
+                                const float pc = 0.5f * (v[zz] - m);
+                                zc[o] = pc;
+                                if constexpr (IDF || DBG) {
+                                    int mid = top ? i2[zz] : i1[zz];
+                                    if (!(m > -eps)) mid = -1;
+                                    if (IDF) B.IDF[oc + o] = mid;
+                                    if (DBG) {
+                                        dbg.m[oc + o] = m;
+                                        dbg.idm[oc + o] = mid;
+                                        dbg.phic[oc + o] = pc;
+                                        dbg.phip[oc + o] = v[zz];
+                                    }
+                                }
+                            }
+                        }
+                    };
                     if (zaff >> 31) {                   // affine (uniform across the CTA)
                         if (!((t.xmask >> lx) & (t.ymask >> ly) & 1u)) continue;
-                        const long long oc = t.off + (long long)(ly * t.nx + lx);
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) o[zz] = oc + (long long)zz * ps;
+                        cells(t.off + (long long)(ly * t.nx + lx), [](int zz) { return zz; });
                     } else {
                         if (!zm) continue;
                         int bxl = t.dx + lx, byl = t.dy + ly;
                         if (bxl >= D.nx) bxl -= D.nx;
                         if (byl >= D.ny) byl -= D.ny;
                         if (bxl >= t.nx || byl >= t.ny) continue;
-                        const long long oc = t.off + (long long)byl * t.nx + bxl;
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) {
-                            int lz = t.dz + zz;
-                            if (lz >= D.nz) lz -= D.nz;
-                            o[zz] = oc + (long long)lz * ps;
-                        }
-                    }
-                    float v[kTileZ];
-                    if (zm == 0xffu) {                  // the whole column (uniform)
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) v[zz] = B.Y[o[zz]];
-                    } else {
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) v[zz] = (zm >> zz) & 1u ? B.Y[o[zz]] : -INFINITY;
-                    }
-                    if (sweep == 0) {
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) top2_insert(v[zz], id, v1[zz], i1[zz], v2[zz], i2[zz]);
-                    } else {
-#pragma unroll
-                        for (int zz = 0; zz < kTileZ; ++zz) {
-                            if (!((zm >> zz) & 1u)) continue;
-                            const bool top = i1[zz] == id;
-                            const float m = top ? w2[zz] : w1[zz];
-                            const float pc = 0.5f * (v[zz] - m);
-                            B.Z[o[zz]] = pc;
-                            if (IDF || DBG) {
-                                int mid = top ? i2[zz] : i1[zz];
-                                if (!(m > -eps)) mid = -1;
-                                if (IDF) B.IDF[o[zz]] = mid;
-                                if (DBG) {
-                                    dbg.m[o[zz]] = m;
-                                    dbg.idm[o[zz]] = mid;
-                                    dbg.phic[o[zz]] = pc;
-                                    dbg.phip[o[zz]] = v[zz];
-                                }
-                            }
-                        }
+                        const int dz = t.dz, dnz = D.nz;
+                        cells(t.off + (long long)byl * t.nx + bxl, [dz, dnz](int zz) {
+                            const int lz = dz + zz;
+                            return lz >= dnz ? lz - dnz : lz;
+                        });
                     }
                 }
             }
@@ -2017,10 +2062,10 @@ cudaError_t configure_passes(StepBuffers& B) {
         }
     }
     int of = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, false>, kTileX * kTileY, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, false, false>, kTileX * kTileY, 0);
     if (e != cudaSuccess) return e;
     B.field_grid[0] = B.n_sm * (of < 1 ? 1 : of);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<true, false, false>, kTileX * kTileY, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<true, true, false, false>, kTileX * kTileY, 0);
     if (e != cudaSuccess) return e;
     B.field_grid[1] = B.n_sm * (of < 1 ? 1 : of);
     B.bin_grid = B.n_sm;
@@ -2081,9 +2126,12 @@ cudaError_t launch_bin(const StepBuffers& B, cudaStream_t s) {
 
 cudaError_t launch_field(const StepBuffers& B, const PhysicsDev& phys, const DebugOut& dbg, cudaStream_t s) {
     const bool idf = phys.kind != LSGG_PHYSICS_IDEAL, dg = dbg.m != nullptr;
-    auto k = idf ? (dg ? p_field<true, true, false> : p_field<true, false, false>)
-                 : (dg ? p_field<false, true, false> : p_field<false, false, false>);
-    k<<<B.field_grid[idf || dg ? 1 : 0], kTileX * kTileY, 0, s>>>(B, GroupRef{nullptr, 0}, phys, dbg);
+    const bool ids = idf || dg || B.keep_field;
+    auto k = idf   ? (dg ? p_field<true, true, true, false> : p_field<true, true, false, false>)
+             : dg  ? p_field<true, false, true, false>
+             : ids ? p_field<true, false, false, false>
+                   : p_field<false, false, false, false>;
+    k<<<B.field_grid[ids ? 1 : 0], kTileX * kTileY, 0, s>>>(B, GroupRef{nullptr, 0}, phys, dbg);
     return cudaGetLastError();
 }
 
@@ -2092,7 +2140,7 @@ cudaError_t launch_field(const StepBuffers& B, const PhysicsDev& phys, const Deb
 // variants keep more registers than the single-context ones).
 struct GroupShapes {
     int pgrid[kTiers][5];             // as StepBuffers::pgrid (index 2 unused)
-    int field, bin, n_sm;
+    int field[2], bin, n_sm;           // field grid: values only / with the top two's grains
 };
 static GroupShapes g_group_shapes{};
 
@@ -2152,9 +2200,12 @@ cudaError_t configure_group_kernels(int n_sm) {
         for (int k = 0; k < 5; ++k) sh.pgrid[t][k] = n_sm * (o[k] < 1 ? 1 : o[k]);
     }
     int of = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, true>, kTileX * kTileY, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, false, true>, kTileX * kTileY, 0);
     if (e != cudaSuccess) return e;
-    sh.field = n_sm * (of < 1 ? 1 : of);
+    sh.field[0] = n_sm * (of < 1 ? 1 : of);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<true, false, false, true>, kTileX * kTileY, 0);
+    if (e != cudaSuccess) return e;
+    sh.field[1] = n_sm * (of < 1 ? 1 : of);
     sh.bin = n_sm;
     g_group_shapes = sh;
     return cudaSuccess;
@@ -2168,8 +2219,10 @@ cudaError_t launch_bin_group(const StepBuffers& B0, const GroupRef& grp, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t launch_field_group(const StepBuffers& B0, const GroupRef& grp, cudaStream_t s) {
-    p_field<false, false, true><<<g_group_shapes.field, kTileX * kTileY, 0, s>>>(B0, grp, PhysicsDev{}, DebugOut{});
+// ids: a member stores the field (lsgg_keep_field)
+cudaError_t launch_field_group(const StepBuffers& B0, const GroupRef& grp, bool ids, cudaStream_t s) {
+    auto k = ids ? p_field<true, false, false, true> : p_field<false, false, false, true>;
+    k<<<g_group_shapes.field[ids ? 1 : 0], kTileX * kTileY, 0, s>>>(B0, grp, PhysicsDev{}, DebugOut{});
     return cudaGetLastError();
 }
 

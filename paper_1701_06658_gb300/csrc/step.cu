@@ -1131,7 +1131,7 @@ cudaError_t launch_group_limits(const GroupRef& grp, const long long* lim, cudaS
 // re-initialisation, the pass path): the same kernels as launch_step's pass
 // path, each launched once over all members.  With side streams the binning
 // runs beside the convolution passes and tiers 1.. beside tier 0.
-cudaError_t launch_group_step(const StepBuffers& B0, const GroupRef& grp, const Taps& taps, cudaStream_t s,
+cudaError_t launch_group_step(const StepBuffers& B0, const GroupRef& grp, const Taps& taps, bool keep, cudaStream_t s,
                               const StepStreams* ss) {
     cudaStream_t bs = ss ? ss->side[kTiers - 1] : s;
     cudaError_t e = cudaSuccess;
@@ -1171,7 +1171,7 @@ cudaError_t launch_group_step(const StepBuffers& B0, const GroupRef& grp, const 
         e = traced(cudaStreamWaitEvent(s, ss->join[kTiers - 1], 0), "join wait");
         if (e != cudaSuccess) return e;
     }
-    e = traced(launch_field_group(B0, grp, s), "group field pass");
+    e = traced(launch_field_group(B0, grp, keep, s), "group field pass");
     if (e == cudaSuccess) e = tiers(1);
     if (e != cudaSuccess) return e;
     k_bu_new<true><<<4 * B0.n_sm, kBuChunk, 0, s>>>(B0, grp);

@@ -1,0 +1,65 @@
+"""GPU tests of the pass kernels' variants: a variant chosen by a rule gives,
+bit for bit, what the general form gives on the same state."""
+import numpy as np
+import pytest
+
+from paper_1701_06658_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_1701_06658_gb300 import lsgg
+    lsgg.lib()
+    return lsgg
+
+
+def lattice_seeds(n, k):
+    """k^3 seeds on a cubic lattice: neighbouring functions are equal, to the bit, on the mid-planes."""
+    a = (np.arange(k) + 0.5) * n / k
+    return np.stack(np.meshgrid(a, a, a, indexing="ij"), -1).reshape(-1, 3)
+
+
+def same_state(a, b):
+    pa, pb = a.phi(), b.phi()
+    assert (a.boxes() == b.boxes()).all()
+    assert all(np.array_equal(pa[g], pb[g]) for g in pa) and pa.keys() == pb.keys()
+
+
+@pytest.mark.parametrize("dims,seeds", [
+    ((64, 64, 64), I.voronoi_seeds(5, 60, (64, 64, 64))),
+    ((41, 27, 53), I.voronoi_seeds(6, 20, (41, 27, 53))),        # ragged tiles, boxes across full axes
+    ((48, 48, 48), lattice_seeds(48, 3)),                        # exact ties
+])
+def test_field_pass_without_grains_equals_the_one_with(L, dims, seeds):
+    G = len(seeds)
+    with L.Microstructure(*dims, G, seeds=seeds) as a, L.Microstructure(*dims, G, seeds=seeds) as b:
+        L.keep_field(b.ctx, True)                                # the variant that tracks the top two's grains
+        for m in (a, b):
+            m.step(3, 1.0)
+            m.sync()
+        same_state(a, b)
+
+
+def test_group_with_a_member_that_keeps_the_field(L):
+    kw = [((40, 40, 40), 12, 3), ((48, 32, 40), 14, 4)]
+    ms = [L.Microstructure(*d, g, seeds=I.voronoi_seeds(s, g, d)) for d, g, s in kw]
+    alone = [L.Microstructure(*d, g, seeds=I.voronoi_seeds(s, g, d)) for d, g, s in kw]
+    L.keep_field(ms[1].ctx, True)
+    L.keep_field(alone[1].ctx, True)
+    with L.Group(ms) as grp:
+        grp.step(3, 1.0)
+        for m in ms:
+            m.sync()
+        for m in alone:
+            m.step(3, 1.0)
+            m.sync()
+        for a, b in zip(ms, alone):
+            same_state(a, b)
+        assert L.grain_neighbours(ms[1].ctx, kw[1][1]) == L.grain_neighbours(alone[1].ctx, kw[1][1])
+    for m in ms + alone:
+        m.close()
