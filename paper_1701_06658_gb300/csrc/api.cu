@@ -22,13 +22,14 @@ static_assert(lsgg::kTiers == LSGG_PASS_TIERS, "pass-path tiers of the library a
 
 namespace lsgg {
 cudaError_t launch_init(const Domain& D, int G, const SeedBins& bins, const double* d_seeds, const double* d_weights, int* d_labels,
-                        unsigned* d_bits, long long words_per_row, int* d_bb, Box* d_cur, cudaStream_t s);
+                        unsigned* d_bits, long long words_per_row, int* d_bb, int* d_seed_cell, Box* d_cur,
+                        cudaStream_t s);
 cudaError_t launch_label_boxes(const Domain& D, int G, const int* d_labels, unsigned* d_occ, int words, Box* d_cur,
                                cudaStream_t s);
 cudaError_t launch_label_phi(const Domain& D, int G, const Box* d_cur, const int* d_labels, float* Z, cudaStream_t s);
-cudaError_t launch_sdf(const Domain& D, int G, const Box* d_cur, const double* d_seeds, const double* d_weights,
-                       const unsigned* d_bits, long long words_per_row, float* X, int* IDF, int* d_status,
-                       cudaStream_t s);
+cudaError_t launch_sdf(const Domain& D, const int2* d_items, int n_items, int groups, const Box* d_cur,
+                       const double* d_seeds, const double* d_weights, const unsigned* d_bits, long long words_per_row,
+                       float* X, int* IDF, int* d_status, cudaStream_t s);
 cudaError_t launch_grain_stats(const double* vol, int G, int dim, int n_bins, double r_max, double* out,
                                double* hist, cudaStream_t s);
 cudaError_t launch_volumes(const Domain& D, int G, const Box* cur, const Box* prev, const float* X, double* out,
@@ -545,7 +546,7 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     const long long wpr = (G + 31) / 32;
     int* d_labels = nullptr;
     unsigned* d_bits = nullptr;
-    int* d_bb = nullptr;
+    int* d_bb = nullptr;                         // per grain: offset bounds (6), then its seed's cell (3)
     if ((r = dalloc(c, &c->d_seeds, seeds.size())) != LSGG_OK) return bail(r);
     if (!weights.empty() && (r = dalloc(c, &c->d_weights, weights.size())) != LSGG_OK) return bail(r);
     if ((r = dalloc(c, &c->d_boxes, 2 * (size_t)G)) != LSGG_OK) return bail(r);
@@ -560,7 +561,7 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     if ((r = dalloc(c, &c->B.T, 2 * (size_t)ncell)) != LSGG_OK) return bail(r);
     if ((r = dalloc(c, &d_labels, (size_t)ncell)) != LSGG_OK) return bail(r);
     if ((r = dalloc(c, &d_bits, (size_t)G * wpr)) != LSGG_OK) return bail(r);
-    if ((r = dalloc(c, &d_bb, 6 * (size_t)G)) != LSGG_OK) return bail(r);
+    if ((r = dalloc(c, &d_bb, 9 * (size_t)G)) != LSGG_OK) return bail(r);
     if (!energy.empty()) {
         std::vector<float> ef(energy.begin(), energy.end());
         if ((r = dalloc(c, &c->d_energy, (size_t)G)) != LSGG_OK) return bail(r);
@@ -616,6 +617,8 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     long long bin_bytes = 0;
     float4* d_bpts = nullptr;
     int *d_bids = nullptr, *d_bstart = nullptr;
+    int2* d_sdf_items = nullptr;                 // work items of the initial functions
+    long long sdf_bytes = 0;
     unsigned* d_occ = nullptr;                   // label field: per grain and axis the positions it holds
     const int occ_words = (std::max(D.nx, std::max(D.ny, D.nz)) + 31) / 32;
     if (!from_labels) {
@@ -672,7 +675,8 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         if ((r = dalloc(c, &d_occ, (size_t)G * 3 * occ_words)) != LSGG_OK) return bail(r);
         if (launch_label_boxes(D, G, d_labels, d_occ, occ_words, c->B.cur, c->stream) != cudaSuccess)
             return bail(CUDA_FAIL());
-    } else if (launch_init(D, G, bins, c->d_seeds, c->d_weights, d_labels, d_bits, wpr, d_bb, c->B.cur, c->stream) !=
+    } else if (launch_init(D, G, bins, c->d_seeds, c->d_weights, d_labels, d_bits, wpr, d_bb, d_bb + 6 * (size_t)G, c->B.cur,
+                           c->stream) !=
                cudaSuccess) {
         return bail(CUDA_FAIL());
     }
@@ -748,8 +752,24 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
                           c->stream) != cudaSuccess)
             return bail(CUDA_FAIL());
     } else {
-        if (launch_sdf(D, G, c->B.cur, c->d_seeds, c->d_weights, d_bits, wpr, c->B.bf16 ? c->B.Y : c->B.X,
-                       c->B.IDF, &c->B.st->status, c->stream) != cudaSuccess)
+        // work items of the initial functions: (box, first of `groups` groups of
+        // four cells along x), about eight CTAs per SM and at most 4096 groups
+        // (one image of the neighbour table per CTA)
+        long long all = 0;
+        for (const Box& b : hb) all += b.nx > 0 ? (long long)((b.nx + 3) / 4) * b.ny * b.nz : 0;
+        const int groups = (int)std::min(4096LL, std::max(256LL, all / (8LL * c->B.n_sm) / 256 * 256));
+        std::vector<int2> items;
+        for (int b = 0; b < G; ++b) {
+            if (hb[b].nx <= 0) continue;
+            const int n = (hb[b].nx + 3) / 4 * hb[b].ny * hb[b].nz;
+            for (long long q = 0; q < n; q += groups) items.push_back(make_int2(b, (int)q));
+        }
+        if ((r = dalloc(c, &d_sdf_items, items.size())) != LSGG_OK) return bail(r);
+        sdf_bytes = (long long)std::max<size_t>(items.size() * sizeof(int2), 16);
+        if (cudaMemcpyAsync(d_sdf_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, c->stream) !=
+                cudaSuccess ||
+            launch_sdf(D, d_sdf_items, (int)items.size(), groups, c->B.cur, c->d_seeds, c->d_weights, d_bits, wpr,
+                       c->B.bf16 ? c->B.Y : c->B.X, c->B.IDF, &c->B.st->status, c->stream) != cudaSuccess)
             return bail(CUDA_FAIL());
         if (c->B.bf16 && launch_f32_to_state(c->B.Y, c->B.X, c->B.cap, c->stream) != cudaSuccess)
             return bail(CUDA_FAIL());
@@ -769,7 +789,8 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     dfree(c, d_bpts);
     dfree(c, d_bids);
     dfree(c, d_bstart);
-    c->device_bytes -= (long long)ncell * 4 + (long long)G * wpr * 4 + 6LL * G * 4 + bin_bytes;
+    dfree(c, d_sdf_items);
+    c->device_bytes -= (long long)ncell * 4 + (long long)G * wpr * 4 + 9LL * G * 4 + bin_bytes + sdf_bytes;
     *out = c;
     return LSGG_OK;
 }

@@ -3,13 +3,14 @@
 //
 //   k_labels        power-diagram label of each cell: argmin_i |x - s_i|^2 - w_i
 //                   with minimum-image displacements, lowest id on ties.  The
-//                   seeds are binned on a uniform grid; an FP32 search over the
-//                   bins around the cell bounds the minimum, and candidates within
-//                   a safe margin of it are decided in FP64 with explicitly
+//                   seeds are binned on a uniform grid; a CTA takes a tile of
+//                   cells and collects once the seeds that can hold one of them,
+//                   its cells compare those in FP32, and candidates within a safe
+//                   margin of the minimum are decided in FP64 with explicitly
 //                   rounded operations, so the integer result does not depend on
 //                   FMA contraction or on the search order.
-//   k_face_pairs    grains whose cells touch across a face (bit matrix).
-//   k_label_bbox    per grain, min/max of the integer minimum-image offsets of its
+//   k_label_faces   grains whose cells touch across a face (bit matrix); per
+//                   grain, min/max of the integer minimum-image offsets of its
 //                   cells from its rounded seed.
 //   k_init_boxes    box = that bbox grown by the halo (full axis if it reaches N).
 //   k_sdf           phi_i(x) = clamp(min_{j in Nb(i)} signed distance of x to the
@@ -159,55 +160,193 @@ __device__ __forceinline__ int label_cell(const Domain& D, const SeedBins& S, co
     return arg;
 }
 
-__global__ void __launch_bounds__(256)
+// The labels, a CTA per tile of kLabelCells cells (8 x 8 x 8, in 2D 32 x 16).
+// A cell-by-cell search reads every bin within its reach again for every cell,
+// and with weights the reach is that of the largest weight (some thousand
+// seeds a cell): 440 ms at 512^3 / 40 000 weighted seeds, 4.6 ms at 256^3 /
+// 5000 on GB300, against 5.1 and 0.52 ms per tile, bound by the FP32 compares
+// (about eight instructions a cell and candidate).  Per tile the search runs once: an upper bound of the power
+// distance that some seed keeps over the whole tile (from the bins around its
+// centre) leaves the seeds whose smallest distance to the tile does not exceed
+// it, typically 20-60, staged in shared memory with FP32 displacements from the
+// tile's centre (rounded from FP64, so that the FP32 error is that of the
+// displacement and not of the domain's size).  Each cell keeps the smallest
+// and second smallest value; unless they are closer than twice the FP32 error
+// bound the smallest one's seed is the label, otherwise FP64 decides among the
+// candidates within it.  A tile with more than kLabelCand candidates (seeds
+// nearly as dense as cells) takes the cell-by-cell search.
+constexpr int kLabelCells = 512;
+constexpr int kLabelThreads = 256;
+constexpr int kLabelCand = 768;
+
+__global__ void __launch_bounds__(kLabelThreads)
 k_labels(Domain D, int G, SeedBins S, const double* __restrict__ seeds, const double* __restrict__ weights,
-         int* __restrict__ labels) {
-    const long long ncell = (long long)D.nx * D.ny * D.nz;
-    const long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (cell >= ncell) return;
-    labels[cell] = label_cell(D, S, seeds, weights, cell);
-}
-
-// The same labels from a persistent grid whose CTAs first copy the binned
-// seeds (points and bin starts) into shared memory: the search's dependent
-// loads then come from shared memory instead of L2.
-__global__ void __launch_bounds__(512)
-k_labels_staged(Domain D, int G, SeedBins S, long long n_bins, const double* __restrict__ seeds,
-                const double* __restrict__ weights, int* __restrict__ labels) {
-    extern __shared__ __align__(16) unsigned char sm_labels[];
-    float4* s_pts = reinterpret_cast<float4*>(sm_labels);
-    int* s_start = reinterpret_cast<int*>(s_pts + G);
-    for (int i = threadIdx.x; i < G; i += blockDim.x) s_pts[i] = S.pts[i];
-    for (long long i = threadIdx.x; i <= n_bins; i += blockDim.x) s_start[i] = S.start[i];
-    __syncthreads();
-    SeedBins L = S;
-    L.pts = s_pts;
-    L.start = s_start;
-    const long long ncell = (long long)D.nx * D.ny * D.nz;
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < ncell;
-         cell += (long long)gridDim.x * blockDim.x)
-        labels[cell] = label_cell(D, L, seeds, weights, cell);
-}
-
-__global__ void k_face_pairs(Domain D, int G, const int* __restrict__ labels, unsigned* __restrict__ bits,
-                             long long words_per_row) {
-    const long long ncell = (long long)D.nx * D.ny * D.nz;
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < ncell;
-         cell += (long long)gridDim.x * blockDim.x) {
-        int x = (int)(cell % D.nx);
-        int y = (int)((cell / D.nx) % D.ny);
-        int z = (int)(cell / ((long long)D.nx * D.ny));
-        int a = labels[cell];
-        int nbr[3];
-        nbr[0] = labels[((long long)z * D.ny + y) * D.nx + (x + 1) % D.nx];
-        nbr[1] = labels[((long long)z * D.ny + (y + 1) % D.ny) * D.nx + x];
-        nbr[2] = D.dim == 3 ? labels[((long long)((z + 1) % D.nz) * D.ny + y) * D.nx + x] : a;
-        for (int k = 0; k < 3; ++k) {
-            int b = nbr[k];
-            if (b == a) continue;
-            atomicOr(&bits[(long long)a * words_per_row + (b >> 5)], 1u << (b & 31));
-            atomicOr(&bits[(long long)b * words_per_row + (a >> 5)], 1u << (a & 31));
+         int* __restrict__ labels, int tx, int ty, int tz, int ntx, int nty) {
+    __shared__ float4 s_c[kLabelCand];               // displacement from the tile's centre, weight
+    __shared__ int s_q[kLabelCand];                  // sorted seed index
+    __shared__ float s_red[kLabelThreads / 32];
+    __shared__ float s_far;                          // largest squared reach of a candidate
+    __shared__ int s_n, s_wrap;
+    const int t = threadIdx.x;
+    const int bx = blockIdx.x % ntx, by = (blockIdx.x / ntx) % nty, bz = blockIdx.x / (ntx * nty);
+    const int o[3] = {bx * tx, by * ty, bz * tz};
+    const int N[3] = {D.nx, D.ny, D.nz};
+    const float fN[3] = {(float)D.nx, (float)D.ny, (float)D.nz};
+    const int e[3] = {min(tx, D.nx - o[0]), min(ty, D.ny - o[1]), min(tz, D.nz - o[2])};
+    float c[3], h[3];                                // centre and half extent over the cells' points
+    int cb[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        c[a] = (float)o[a] + 0.5f * (float)(e[a] - 1);
+        h[a] = 0.5f * (float)(e[a] - 1);
+        cb[a] = min(S.nb[a] - 1, (int)(c[a] / S.size[a]));
+    }
+    // squared power distances of a seed to the tile: smallest and largest over its cells
+    auto range = [&](const float4 p, float& near, float& far) {
+        const float q[3] = {p.x, p.y, p.z};
+        near = far = -p.w;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float d = fabsf(wrap_half(c[a] - q[a], fN[a]));
+            const float n0 = fmaxf(d - h[a], 0.0f), f0 = fminf(d + h[a], 0.5f * fN[a]);
+            near = fmaf(n0, n0, near);
+            far = fmaf(f0, f0, far);
         }
+    };
+    // the bins [lo, lo + cnt) per axis (cyclic), spread over the threads
+    auto for_bins = [&](const int (&lo)[3], const int (&cnt)[3], auto f) {
+        const int nbin = cnt[0] * cnt[1] * cnt[2];
+        for (int k = t; k < nbin; k += kLabelThreads) {
+            const int ix = k % cnt[0], iy = (k / cnt[0]) % cnt[1], iz = k / (cnt[0] * cnt[1]);
+            const int bin = (wrap_bin(lo[2] + iz, S.nb[2]) * S.nb[1] + wrap_bin(lo[1] + iy, S.nb[1])) * S.nb[0] +
+                            wrap_bin(lo[0] + ix, S.nb[0]);
+            for (int q = S.start[bin]; q < S.start[bin + 1]; ++q) f(q);
+        }
+    };
+    auto block_min = [&](float v) {
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, k));
+        __syncthreads();
+        if ((t & 31) == 0) s_red[t >> 5] = v;
+        __syncthreads();
+        v = s_red[0];
+#pragma unroll
+        for (int k = 1; k < kLabelThreads / 32; ++k) v = fminf(v, s_red[k]);
+        return v;
+    };
+    // an upper bound that one seed keeps over the tile, from the bins around the centre
+    float bound = FLT_MAX;
+    int lo[3], cnt[3];
+    for (int k = 1; bound == FLT_MAX; k *= 2) {
+        bool whole = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            bin_range(cb[a], k, S.nb[a], lo[a], cnt[a]);
+            whole = whole && cnt[a] == S.nb[a];
+        }
+        float m = FLT_MAX;
+        for_bins(lo, cnt, [&](int q) {
+            float near, far;
+            range(S.pts[q], near, far);
+            m = fminf(m, far);
+        });
+        bound = block_min(m);
+        if (whole) break;
+    }
+    const float nmax = fmaxf(fN[0], fmaxf(fN[1], fN[2]));
+    // margin covering FP32 rounding of |d|^2 <= 3 N^2, of the seeds and of the weights
+    bound += 0.5f + 4e-6f * nmax * nmax + 1e-5f * fabsf(bound);
+    // the seeds that can hold a cell lie within r of the tile on every axis
+    const float r = sqrtf(fmaxf(0.0f, bound + S.wmax)) + 1.0f;   // + 1: bin-edge rounding
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float ra = r + h[a];
+        lo[a] = 0;
+        cnt[a] = S.nb[a];
+        if (2.0f * ra + 2.0f * S.size[a] < (float)S.nb[a] * S.size[a]) {
+            const int l = (int)floorf((c[a] - ra) / S.size[a]), u = (int)floorf((c[a] + ra) / S.size[a]);
+            if (u - l + 1 < S.nb[a]) {
+                cnt[a] = u - l + 1;
+                lo[a] = l % S.nb[a];
+                if (lo[a] < 0) lo[a] += S.nb[a];
+            }
+        }
+    }
+    if (t == 0) { s_n = 0; s_wrap = 0; s_far = 0.0f; }
+    __syncthreads();
+    for_bins(lo, cnt, [&](int q) {
+        const float4 p = S.pts[q];
+        float near, far;
+        range(p, near, far);
+        if (near > bound) return;
+        const int k = atomicAdd(&s_n, 1);
+        if (k >= kLabelCand) return;
+        const int i = S.ids[q];
+        float d[3], r2 = 0.0f;
+        bool wrap = false;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            d[a] = (float)min_image(__dsub_rn(seeds[3 * i + a], (double)c[a]), (double)N[a]);
+            const float u = fabsf(d[a]) + h[a];
+            wrap = wrap || (N[a] > 1 && u > 0.5f * fN[a] - 0.01f);
+            r2 = fmaf(u, u, r2);
+        }
+        s_c[k] = make_float4(d[0], d[1], d[2], p.w);
+        s_q[k] = q;
+        if (wrap) s_wrap = 1;
+        atomicMax(reinterpret_cast<int*>(&s_far), __float_as_int(r2 + fabsf(p.w)));   // non-negative floats
+    });
+    __syncthreads();
+    const int n = s_n;
+    const bool wrap = s_wrap != 0;
+    // twice the FP32 error of a candidate's value: displacements and squares
+    // (5e-7 of the squared reach), the weight's rounding and the difference's
+    const float margin = 4e-6f * s_far + 1e-4f;
+    for (int k = t; k < e[0] * e[1] * e[2]; k += kLabelThreads) {
+        const int x = k % e[0], y = (k / e[0]) % e[1], z = k / (e[0] * e[1]);
+        const int g[3] = {o[0] + x, o[1] + y, o[2] + z};
+        const long long cell = ((long long)g[2] * D.ny + g[1]) * D.nx + g[0];
+        if (n > kLabelCand) {
+            labels[cell] = label_cell(D, S, seeds, weights, cell);
+            continue;
+        }
+        const float p[3] = {(float)x - h[0], (float)y - h[1], (float)z - h[2]};
+        auto value = [&](int q) {
+            const float4 s = s_c[q];
+            float dx = p[0] - s.x, dy = p[1] - s.y, dz = p[2] - s.z;
+            if (wrap) {
+                dx = wrap_half(dx, fN[0]);
+                dy = wrap_half(dy, fN[1]);
+                dz = wrap_half(dz, fN[2]);
+            }
+            return fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -s.w)));
+        };
+        float v1 = FLT_MAX, v2 = FLT_MAX;
+        int k1 = 0;
+        for (int q = 0; q < n; ++q) {
+            const float v = value(q);
+            k1 = v < v1 ? q : k1;
+            v2 = fminf(v2, fmaxf(v1, v));
+            v1 = fminf(v1, v);
+        }
+        int arg;
+        if (v2 > v1 + margin) {
+            arg = S.ids[s_q[k1]];
+        } else {
+            double best = DBL_MAX;
+            arg = -1;
+            for (int q = 0; q < n; ++q) {
+                if (value(q) > v1 + margin) continue;
+                const int i = S.ids[s_q[q]];
+                const double ex = min_image(__dsub_rn((double)g[0], seeds[3 * i]), (double)D.nx);
+                const double ey = min_image(__dsub_rn((double)g[1], seeds[3 * i + 1]), (double)D.ny);
+                const double ez = min_image(__dsub_rn((double)g[2], seeds[3 * i + 2]), (double)D.nz);
+                double rr = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
+                if (weights) rr = __dsub_rn(rr, weights[i]);
+                if (rr < best || (rr == best && i < arg)) { best = rr; arg = i; }
+            }
+        }
+        labels[cell] = arg;
     }
 }
 
@@ -216,28 +355,59 @@ __device__ __forceinline__ int offset_from(int x, int r, int n) {
     return e > n / 2 ? e - n : e;
 }
 
-__global__ void k_bbox_init(int G, int* bb) {
+// Per grain: its rounded seed's cell, and empty offset bounds.
+__global__ void k_bbox_init(Domain D, int G, const double* __restrict__ seeds, int* bb, int* seed_cell) {
+    const int N[3] = {D.nx, D.ny, D.nz};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G; i += gridDim.x * blockDim.x) {
-        for (int a = 0; a < 3; ++a) { bb[6 * i + a] = INT_MAX; bb[6 * i + 3 + a] = INT_MIN; }
+        for (int a = 0; a < 3; ++a) {
+            bb[6 * i + a] = INT_MAX;
+            bb[6 * i + 3 + a] = INT_MIN;
+            seed_cell[3 * i + a] = pmod((int)rint(seeds[3 * i + a]), N[a]);
+        }
     }
 }
 
-__global__ void k_label_bbox(Domain D, const int* __restrict__ labels, const double* __restrict__ seeds,
-                             int* __restrict__ bb) {
+__device__ __forceinline__ void set_pair_bit(unsigned* bits, long long words_per_row, int a, int b) {
+    unsigned* w = bits + (long long)a * words_per_row + (b >> 5);
+    const unsigned m = 1u << (b & 31);
+    if (!(*(volatile unsigned*)w & m)) atomicOr(w, m);
+}
+
+// A thread per cell and its next cell on every axis (periodic).  Different
+// labels: the two grains touch, and only such a cell can be the last of its
+// grain on the axis and the next one the first of its own; equal labels count
+// only across the cut of the grain's offsets (half a period from its seed).
+// Taking every cell's offsets took 6 atomics a cell: 14.9 ms with the pairs at
+// 512^3 on GB300, against 2.2 ms.
+__global__ void __launch_bounds__(256)
+k_label_faces(Domain D, const int* __restrict__ labels, const int* __restrict__ seed_cell,
+              unsigned* __restrict__ bits, long long words_per_row, int* __restrict__ bb) {
     const long long ncell = (long long)D.nx * D.ny * D.nz;
+    const int N[3] = {D.nx, D.ny, D.nz};
+    const long long st[3] = {1, D.nx, (long long)D.nx * D.ny};
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < ncell;
          cell += (long long)gridDim.x * blockDim.x) {
-        int x = (int)(cell % D.nx);
-        int y = (int)((cell / D.nx) % D.ny);
-        int z = (int)(cell / ((long long)D.nx * D.ny));
-        int i = labels[cell];
-        int c[3] = {x, y, z};
-        int N[3] = {D.nx, D.ny, D.nz};
-        for (int a = 0; a < 3; ++a) {
-            int r = pmod((int)rint(seeds[3 * i + a]), N[a]);
-            int e = offset_from(c[a], r, N[a]);
-            atomicMin(&bb[6 * i + a], e);
-            atomicMax(&bb[6 * i + 3 + a], e);
+        const int c[3] = {(int)(cell % D.nx), (int)((cell / D.nx) % D.ny), (int)(cell / ((long long)D.nx * D.ny))};
+        const int a = labels[cell];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (N[k] == 1) continue;
+            const int nx = c[k] + 1 < N[k] ? c[k] + 1 : 0;
+            const int b = labels[cell + (long long)(nx - c[k]) * st[k]];
+            const int ra = seed_cell[3 * a + k];
+            if (b != a) {
+                set_pair_bit(bits, words_per_row, a, b);
+                set_pair_bit(bits, words_per_row, b, a);
+                atomicMax(&bb[6 * a + 3 + k], offset_from(c[k], ra, N[k]));
+                atomicMin(&bb[6 * b + k], offset_from(nx, seed_cell[3 * b + k], N[k]));
+            } else {
+                int cut = ra + N[k] / 2 + 1;          // the first cell past half a period
+                if (cut >= N[k]) cut -= N[k];
+                if (nx == cut) {
+                    atomicMax(&bb[6 * a + 3 + k], offset_from(c[k], ra, N[k]));
+                    atomicMin(&bb[6 * a + k], offset_from(nx, ra, N[k]));
+                }
+            }
         }
     }
 }
@@ -266,6 +436,7 @@ __global__ void k_init_boxes(Domain D, int G, const int* __restrict__ bb, const 
     }
 }
 
+// neighbours of a grain the initial functions take (more: refused)
 constexpr int kSdfNb = 512;
 
 __device__ __forceinline__ double power_dist(const double* p, const double* s, double w, const double* N,
@@ -293,45 +464,106 @@ struct SdfPair {
     double n0, n1, n2, c;
 };
 
-__global__ void __launch_bounds__(256)
-k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__ seeds,
-      const double* __restrict__ weights, const unsigned* __restrict__ bits, long long words_per_row,
-      float* __restrict__ X, int* __restrict__ IDF, int* __restrict__ status) {
+__device__ __forceinline__ float two_sum_f(float a, float b, float& e) {
+    const float s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
+constexpr int kSdfThreads = 256;
+
+// A CTA per item (box, first of `groups` groups of four cells along x).  One
+// CTA a box leaves a large grain's box (hundreds of neighbours, 10^6 cells) on
+// one SM: 130 ms of a 160^3 lognormal start on GB300, 176 ms at 512^3; the
+// items below take 3.6 and 15.5 ms, bound by the screening's issue slots.
+//
+// Where every cell of the box sees the seed and every neighbour through one
+// image (any box small against the domain) the values are affine throughout
+// (`fast`): a thread screens a group of four cells at once, the two smallest
+// FP32 values of each kept in registers (six instructions a cell and neighbour).
+// With the smallest one clear of the other by twice the FP32 error bound E, its
+// value is taken in double-float arithmetic (pairs of FP32, about 2^-47 of the
+// terms' size), and it is the FP64 value's FP32 rounding unless a rounding
+// boundary lies within that error; then, and where E does not separate the two,
+// the cell takes the general FP64 form (`slow_cell`), as every cell of a box
+// without `fast` does.  FP64 for every cell's winner kept the FP64 pipe busy:
+// 9.6 ms at 256^3 / 5000 grains, against 1.95 ms.
+__global__ void __launch_bounds__(kSdfThreads)
+k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restrict__ boxes,
+      const double* __restrict__ seeds, const double* __restrict__ weights, const unsigned* __restrict__ bits,
+      long long words_per_row, float* __restrict__ X, int* __restrict__ IDF, int* __restrict__ status) {
     __shared__ int s_nb[kSdfNb];
     __shared__ float4 s_d[kSdfNb];          // D = s_i - s_j (minimum image), w_j - w_i
     __shared__ float4 s_f[kSdfNb];          // n and c in FP32
+    __shared__ float4 s_l[kSdfNb];          // what FP32 leaves of them
     __shared__ SdfPair s_p[kSdfNb];         // n and c in FP64
-    __shared__ int s_cnt;
-    const int i = blockIdx.x;
+    __shared__ int s_warp[kSdfThreads / 32];
+    __shared__ float s_cmax;
+    const int i = items[blockIdx.x].x;
     const Box b = boxes[i];
-    if (b.nx <= 0) return;
-    if (threadIdx.x == 0) {
-        int cnt = 0;
-        for (long long w = 0; w < words_per_row; ++w) {
-            unsigned m = bits[(long long)i * words_per_row + w];
-            while (m) {
-                int bit = __ffs(m) - 1;
-                m &= m - 1;
-                if (cnt < kSdfNb) s_nb[cnt] = (int)(w * 32 + bit);
-                ++cnt;
-            }
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // the neighbours in ascending order: a word of the bit row per thread, its
+    // bits placed by a block-wide prefix of the counts
+    int cnt = 0;
+    for (long long w0 = 0; w0 < words_per_row; w0 += kSdfThreads) {
+        unsigned m = w0 + t < words_per_row ? bits[(long long)i * words_per_row + w0 + t] : 0u;
+        const int own = __popc(m);
+        int pre = own;
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pre, k);
+            if (lane >= k) pre += v;
         }
-        if (cnt > kSdfNb) { atomicExch(status, -8); cnt = kSdfNb; }
-        s_cnt = cnt;
+        if (lane == 31) s_warp[warp] = pre;
+        __syncthreads();
+        int at = cnt + pre - own, total = 0;
+#pragma unroll
+        for (int k = 0; k < kSdfThreads / 32; ++k) {
+            if (k < warp) at += s_warp[k];
+            total += s_warp[k];
+        }
+        for (; m; m &= m - 1, ++at)
+            if (at < kSdfNb) s_nb[at] = (int)((w0 + t) * 32 + __ffs(m) - 1);
+        cnt += total;
+        __syncthreads();
     }
+    if (cnt > kSdfNb) {
+        if (t == 0) atomicExch(status, -8);
+        cnt = kSdfNb;
+    }
+    if (t == 0) s_cmax = 0.0f;
     __syncthreads();
-    const int cnt = s_cnt;
     const double si[3] = {seeds[3 * i], seeds[3 * i + 1], seeds[3 * i + 2]};
     const double wi = weights ? weights[i] : 0.0;
     const double Nd[3] = {(double)D.nx, (double)D.ny, (double)D.nz};
     const float Nf[3] = {(float)D.nx, (float)D.ny, (float)D.nz};
     const int Ni[3] = {D.nx, D.ny, D.nz};
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+    const int o[3] = {b.ox, b.oy, b.oz};
+    const int bn[3] = {b.nx, b.ny, b.nz};
+    // the box's cells as consecutive integers q = shift + l whose displacement
+    // q - s_i stays within half a period (fast), its first and last values
+    int shift[3];
+    float first[3], last[3], asum = 0.0f;
+    bool fast = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        shift[a] = o[a];
+        const double d0 = (double)o[a] - si[a];
+        if (d0 > 0.5 * Nd[a]) shift[a] -= Ni[a];
+        else if (d0 < -0.5 * Nd[a]) shift[a] += Ni[a];
+        first[a] = (float)((double)shift[a] - si[a]);
+        last[a] = first[a] + (float)(bn[a] - 1);
+        fast = fast && first[a] > -0.5f * Nf[a] + 2e-2f && last[a] < 0.5f * Nf[a] - 2e-2f && Ni[a] < (1 << 22);
+        asum += fmaxf(fabsf(first[a]), fabsf(last[a]));
+    }
+    for (int k = t; k < cnt; k += kSdfThreads) {
         const int j = s_nb[k];
         const double wj = weights ? weights[j] : 0.0;
         const double d0 = min_image(si[0] - seeds[3 * j], Nd[0]), d1 = min_image(si[1] - seeds[3 * j + 1], Nd[1]),
                      d2 = min_image(si[2] - seeds[3 * j + 2], Nd[2]);
-        s_d[k] = make_float4((float)d0, (float)d1, (float)d2, (float)(wj - wi));
+        const float df[3] = {(float)d0, (float)d1, (float)d2};
+        s_d[k] = make_float4(df[0], df[1], df[2], (float)(wj - wi));
         const double len = sqrt(fma(d0, d0, fma(d1, d1, d2 * d2)));
         SdfPair q;
         q.n0 = d0 / len;
@@ -339,21 +571,25 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
         q.n2 = d2 / len;
         q.c = 0.5 * len - 0.5 * (wj - wi) / len;
         s_p[k] = q;
-        s_f[k] = make_float4((float)q.n0, (float)q.n1, (float)q.n2, (float)q.c);
+        const float4 f = make_float4((float)q.n0, (float)q.n1, (float)q.n2, (float)q.c);
+        s_f[k] = f;
+        s_l[k] = make_float4((float)(q.n0 - (double)f.x), (float)(q.n1 - (double)f.y), (float)(q.n2 - (double)f.z),
+                             (float)(q.c - (double)f.w));
+        // one image of the neighbour's seed for every cell of the box
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            fast = fast && fabsf(first[a] + df[a]) < 0.5f * Nf[a] - 2e-2f && fabsf(last[a] + df[a]) < 0.5f * Nf[a] - 2e-2f;
+        fast = fast && fabsf(f.w) < 1e6f;
+        atomicMax(reinterpret_cast<int*>(&s_cmax), __float_as_int(fabsf(f.w)));
     }
-    __syncthreads();
+    fast = __syncthreads_and(fast);
     const float sif[3] = {(float)si[0], (float)si[1], (float)si[2]};
     const float nmax = fmaxf(Nf[0], fmaxf(Nf[1], Nf[2]));
-    const int A = b.nx * b.ny;
     const int ps = plane_stride(b.nx, b.ny);
-    const int ncell = A * b.nz;
     const double eps = (double)D.eps;
-    const int o[3] = {b.ox, b.oy, b.oz};
-    for (int idx = threadIdx.x; idx < ncell; idx += blockDim.x) {
-        const int z = idx / A;
-        const int rem = idx - z * A;
-        const int y = rem / b.nx, x = rem - y * b.nx;
-        const int l[3] = {x, y, z};
+
+    // the general form at the box's cell l (local coordinates): value and neighbour
+    auto slow_cell = [&](const int (&l)[3], int& arg) {
         // the cell's global coordinates g and its displacement from s_i: the
         // image decided in FP32 (g - (float)s_i is exact), FP64 only for the value
         int g[3], sh[3];
@@ -382,15 +618,15 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
             a1 = __dsub_rn((double)(g[1] + sh[1]), si[1]);
             a2 = __dsub_rn((double)(g[2] + sh[2]), si[2]);
         }
-        const float asum = fabsf(af[0]) + fabsf(af[1]) + fabsf(af[2]);
+        const float as = fabsf(af[0]) + fabsf(af[1]) + fabsf(af[2]);
         // whether neighbour k's image for this cell is D's (then the affine form
         // holds); near half a period the general form decides
         auto affine = [&](const float4& dk) {
             bool ok = !amb;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float t = af[c] + (c == 0 ? dk.x : (c == 1 ? dk.y : dk.z));
-                ok &= fabsf(t) < 0.5f * Nf[c] - 1e-2f;
+                const float v = af[c] + (c == 0 ? dk.x : (c == 1 ? dk.y : dk.z));
+                ok &= fabsf(v) < 0.5f * Nf[c] - 1e-2f;
             }
             return ok;
         };
@@ -400,7 +636,7 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
                 const float4 f = s_f[k];
                 v = fmaf(f.x, af[0], fmaf(f.y, af[1], fmaf(f.z, af[2], f.w)));
                 // rounding of s_i, n and c to FP32 and of the three FMAs
-                err = 2.4e-7f * (3.0f * nmax + 2.0f * asum + 2.0f * fabsf(f.w) + 4.0f);
+                err = 2.4e-7f * (3.0f * nmax + 2.0f * as + 2.0f * fabsf(f.w) + 4.0f);
                 return;
             }
             const float dd[3] = {dk.x, dk.y, dk.z};
@@ -408,9 +644,9 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
             bool near_half = false;                            // image choice too close to call in FP32
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float t = af[c] + dd[c];                 // p - s_j before wrapping
-                near_half |= fabsf(fabsf(t) - 0.5f * Nf[c]) < 1e-2f;
-                const float dc = t > 0.5f * Nf[c] ? dd[c] - Nf[c] : (t < -0.5f * Nf[c] ? dd[c] + Nf[c] : dd[c]);
+                const float u = af[c] + dd[c];                 // p - s_j before wrapping
+                near_half |= fabsf(fabsf(u) - 0.5f * Nf[c]) < 1e-2f;
+                const float dc = u > 0.5f * Nf[c] ? dd[c] - Nf[c] : (u < -0.5f * Nf[c] ? dd[c] + Nf[c] : dd[c]);
                 num = fmaf(dc, fmaf(2.0f, af[c], dc), num);
                 den = fmaf(dc, dc, den);
             }
@@ -418,29 +654,23 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
             v = 0.5f * num * rinv;
             // about 64 FP32 ulps of every term of num / (2 |d|), and of v
             err = near_half || amb ? FLT_MAX
-                                   : 4e-6f * (0.5f * den * rinv + asum + 0.5f * fabsf(dk.w) * rinv + fabsf(v) + 1.0f);
+                                   : 4e-6f * (0.5f * den * rinv + as + 0.5f * fabsf(dk.w) * rinv + fabsf(v) + 1.0f);
         };
-        // one screening pass keeps the neighbours that may still be the minimum
-        // (v - err <= the running bound U); a full list falls back to a rescan
-        constexpr int kCand = 6;
-        int cand[kCand];
-        float cand_lo[kCand];
-        int n_cand = 0;
-        bool rescan = false;
+        // the screening's upper bound U of the minimum, then the exact
+        // evaluation of the neighbours that may be it, in neighbour order (which
+        // decides ties, as in the definition)
         float U = FLT_MAX;
         for (int k = 0; k < cnt; ++k) {
             float v, err;
             screen(k, v, err);
             U = fminf(U, v + err);
-            if (v - err <= U) {
-                if (n_cand < kCand) { cand[n_cand] = k; cand_lo[n_cand] = v - err; ++n_cand; }
-                else rescan = true;
-            }
         }
-        // exact evaluation of the candidates (neighbour order decides ties, as in the definition)
         double best = DBL_MAX;
-        int arg = -1;
-        auto exact = [&](int k) {
+        arg = -1;
+        for (int k = 0; k < cnt; ++k) {
+            float v, err;
+            screen(k, v, err);
+            if (!(v - err <= U)) continue;
             const int j = s_nb[k];
             double ve;
             if (affine(s_d[k])) {
@@ -457,55 +687,114 @@ k_sdf(Domain D, int G, const Box* __restrict__ boxes, const double* __restrict__
                 ve = num * (0.5 * rsqrt(fma(d0, d0, fma(d1, d1, d2 * d2))));
             }
             if (ve < best) { best = ve; arg = j; }
-        };
-        if (!rescan) {
-            for (int q = 0; q < n_cand; ++q)           // ascending neighbour order
-                if (cand_lo[q] <= U) exact(cand[q]);
-        } else {
-            for (int k = 0; k < cnt; ++k) {
-                float v, err;
-                screen(k, v, err);
-                if (v - err <= U) exact(k);
+        }
+        return (float)(best == DBL_MAX ? eps : (best < -eps ? -eps : (best > eps ? eps : best)));
+    };
+
+    // FP32 screening error: n and a rounded, three FMAs; double-float error:
+    // s_i to 48 bits, the products' and sums' last places, and the FP64 form's own
+    const float E = 1.2e-7f * (5.0f * asum + 4.0f * s_cmax + 1.0f);
+    const float edd = 1e-14f * (nmax + 2.0f * asum + 2.0f * s_cmax + 2.0f);
+    float s_hi[3], s_lo[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        s_hi[a] = (float)si[a];
+        s_lo[a] = (float)(si[a] - (double)s_hi[a]);
+    }
+    const int ngx = (b.nx + 3) >> 2;
+    const int per_plane = ngx * b.ny;
+    const int g0 = items[blockIdx.x].y, g1 = min(per_plane * b.nz, g0 + groups);
+    for (int q = g0 + t; q < g1; q += kSdfThreads) {
+        const int z = q / per_plane, rem = q - z * per_plane;
+        const int y = rem / ngx, x0 = 4 * (rem - y * ngx);
+        const long long off = b.off + (long long)z * ps + (long long)y * b.nx + x0;
+        if (!fast) {
+            for (int u = 0; u < min(4, b.nx - x0); ++u) {
+                const int l[3] = {x0 + u, y, z};
+                int arg;
+                X[off + u] = slow_cell(l, arg);
+                if (IDF) IDF[off + u] = arg;
+            }
+            continue;
+        }
+        // displacements a = (shift + l) - s_i as pairs (the y and z ones shared)
+        float ah[3], al[3], a0h[4], a0l[4];
+#pragma unroll
+        for (int a = 1; a < 3; ++a) {
+            float e;
+            ah[a] = two_sum_f((float)(shift[a] + (a == 1 ? y : z)), -s_hi[a], e);
+            al[a] = e - s_lo[a];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float e;
+            a0h[u] = two_sum_f((float)(shift[0] + x0 + u), -s_hi[0], e);
+            a0l[u] = e - s_lo[0];
+        }
+        float v1[4], v2[4];
+        int k1[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { v1[u] = v2[u] = FLT_MAX; k1[u] = 0; }
+        for (int k = 0; k < cnt; ++k) {
+            const float4 f = s_f[k];
+            const float row = fmaf(f.y, ah[1], fmaf(f.z, ah[2], f.w));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float v = fmaf(f.x, a0h[u], row);
+                k1[u] = v < v1[u] ? k : k1[u];
+                v2[u] = fminf(v2[u], fmaxf(v1[u], v));
+                v1[u] = fminf(v1[u], v);
             }
         }
-        const double outv = best == DBL_MAX ? eps : (best < -eps ? -eps : (best > eps ? eps : best));
-        const long long off = b.off + (long long)z * ps + rem;
-        X[off] = (float)outv;
-        if (IDF) IDF[off] = arg;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (x0 + u >= b.nx) break;
+            float out = D.eps;
+            int arg = -1;
+            if (cnt > 0) {
+                const float4 f = s_f[k1[u]], lo = s_l[k1[u]];
+                // n . a + c: products exact as pairs, their sum by two-sums
+                const float p0 = f.x * a0h[u], p1 = f.y * ah[1], p2 = f.z * ah[2];
+                float e = fmaf(f.x, a0h[u], -p0) + fmaf(f.y, ah[1], -p1) + fmaf(f.z, ah[2], -p2);
+                e = fmaf(f.x, a0l[u], fmaf(lo.x, a0h[u], e));
+                e = fmaf(f.y, al[1], fmaf(lo.y, ah[1], e));
+                e = fmaf(f.z, al[2], fmaf(lo.z, ah[2], e));
+                float r0, r1, r2;
+                float sum = two_sum_f(p0, p1, r0);
+                sum = two_sum_f(sum, p2, r1);
+                sum = two_sum_f(sum, f.w, r2);
+                e += lo.w + (r0 + r1 + r2);
+                const float hi = __fadd_rn(sum, e), rest = __fsub_rn(e, __fsub_rn(hi, sum));
+                // the nearest FP32 number of every value within edd
+                const bool sure = v2[u] > v1[u] + 2.0f * E && __fadd_rn(hi, rest + edd) == hi &&
+                                  __fadd_rn(hi, rest - edd) == hi;
+                if (sure) {
+                    out = fminf(fmaxf(hi, -D.eps), D.eps);
+                    arg = s_nb[k1[u]];
+                } else {
+                    const int l[3] = {x0 + u, y, z};
+                    out = slow_cell(l, arg);
+                }
+            }
+            X[off + u] = out;
+            if (IDF) IDF[off + u] = arg;
+        }
     }
 }
 
 cudaError_t launch_init(const Domain& D, int G, const SeedBins& bins, const double* d_seeds, const double* d_weights,
-                        int* d_labels, unsigned* d_bits, long long words_per_row, int* d_bb,
+                        int* d_labels, unsigned* d_bits, long long words_per_row, int* d_bb, int* d_seed_cell,
                         Box* d_cur, cudaStream_t s) {
     const long long ncell = (long long)D.nx * D.ny * D.nz;
-    // the binned seeds in shared memory when they fit, else read from global memory
-    const long long n_bins = (long long)bins.nb[0] * bins.nb[1] * bins.nb[2];
-    const size_t staged = (size_t)G * sizeof(float4) + (size_t)(n_bins + 1) * sizeof(int);
-    int dev = 0, n_sm = 0, optin = 0, occ = 0;
-    bool use_staged = cudaGetDevice(&dev) == cudaSuccess &&
-                      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-                      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-                      staged <= (size_t)optin &&
-                      cudaFuncSetAttribute(k_labels_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)staged) == cudaSuccess &&
-                      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_labels_staged, 512, staged) ==
-                          cudaSuccess &&
-                      occ > 0;
-    if (use_staged) {
-        k_labels_staged<<<n_sm * occ, 512, staged, s>>>(D, G, bins, n_bins, d_seeds, d_weights, d_labels);
-    } else {
-        cudaGetLastError();                      // a refused attribute leaves no error behind
-        int blocks = (int)((ncell + 255) / 256);
-        k_labels<<<blocks, 256, 0, s>>>(D, G, bins, d_seeds, d_weights, d_labels);
-    }
+    const int tx = D.dim == 3 ? 8 : 32, ty = D.dim == 3 ? 8 : 16, tz = D.dim == 3 ? 8 : 1;
+    const int ntx = (D.nx + tx - 1) / tx, nty = (D.ny + ty - 1) / ty, ntz = (D.nz + tz - 1) / tz;
+    k_labels<<<ntx * nty * ntz, kLabelThreads, 0, s>>>(D, G, bins, d_seeds, d_weights, d_labels, tx, ty, tz, ntx, nty);
     cudaError_t e = cudaMemsetAsync(d_bits, 0, (size_t)G * words_per_row * 4, s);
     if (e != cudaSuccess) return e;
-    int gs = (int)((ncell + 255) / 256);
+    long long gs = (ncell + 255) / 256;
     if (gs > 65535 * 8) gs = 65535 * 8;
-    k_face_pairs<<<gs, 256, 0, s>>>(D, G, d_labels, d_bits, words_per_row);
-    k_bbox_init<<<(G + 255) / 256, 256, 0, s>>>(G, d_bb);
-    k_label_bbox<<<gs, 256, 0, s>>>(D, d_labels, d_seeds, d_bb);
+    k_bbox_init<<<(G + 255) / 256, 256, 0, s>>>(D, G, d_seeds, d_bb, d_seed_cell);
+    k_label_faces<<<(int)gs, 256, 0, s>>>(D, d_labels, d_seed_cell, d_bits, words_per_row, d_bb);
     k_init_boxes<<<(G + 255) / 256, 256, 0, s>>>(D, G, d_bb, d_seeds, d_cur);
     return cudaGetLastError();
 }
@@ -605,10 +894,12 @@ cudaError_t launch_label_phi(const Domain& D, int G, const Box* d_cur, const int
     return cudaGetLastError();
 }
 
-cudaError_t launch_sdf(const Domain& D, int G, const Box* d_cur, const double* d_seeds, const double* d_weights,
-                       const unsigned* d_bits, long long words_per_row, float* X, int* IDF, int* d_status,
-                       cudaStream_t s) {
-    k_sdf<<<G, 256, 0, s>>>(D, G, d_cur, d_seeds, d_weights, d_bits, words_per_row, X, IDF, d_status);
+cudaError_t launch_sdf(const Domain& D, const int2* d_items, int n_items, int groups, const Box* d_cur,
+                       const double* d_seeds, const double* d_weights, const unsigned* d_bits, long long words_per_row,
+                       float* X, int* IDF, int* d_status, cudaStream_t s) {
+    if (n_items > 0)
+        k_sdf<<<n_items, kSdfThreads, 0, s>>>(D, d_items, groups, d_cur, d_seeds, d_weights, d_bits, words_per_row, X,
+                                              IDF, d_status);
     return cudaGetLastError();
 }
 

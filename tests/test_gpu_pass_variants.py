@@ -63,3 +63,31 @@ def test_group_with_a_member_that_keeps_the_field(L):
         assert L.grain_neighbours(ms[1].ctx, kw[1][1]) == L.grain_neighbours(alone[1].ctx, kw[1][1])
     for m in ms + alone:
         m.close()
+
+
+@pytest.mark.parametrize("dims,G,big", [
+    ((72, 72, 72), 250, 0.0),        # boxes small against the domain: one image per neighbour
+    ((41, 27, 53), 20, 0.0),         # ragged tiles, several images
+    ((16, 16, 16), 1500, 0.0),       # more seeds than a tile's list holds
+    ((40, 40, 48), 90, 300.0),       # power diagram with one grain over most of the domain
+    ((70, 45, 1), 60, 0.0),          # 2D tiles
+])
+def test_start_from_seeds_against_the_oracle(L, dims, G, big):
+    """Boxes equal, functions the FP32 rounding of the oracle's FP64 ones (whose own rounding, about 1e-13 of
+    values up to 7, can move a value across a rounding boundary: one unit in the last place)."""
+    from oracle import lsgg_oracle as O
+    seeds = I.voronoi_seeds(17, G, dims)
+    w = None
+    if big:
+        w = np.zeros(G)
+        w[3] = big
+    ref = O.tessellate((dims[2], dims[1], dims[0]), seeds, w)
+    with L.Microstructure(*dims, G, seeds=seeds, weights=w) as ms:
+        boxes, phi = ms.boxes(), ms.phi()
+    for g, r in enumerate(ref.grains):
+        assert bool(boxes[g, 0]) == r.alive
+        if not r.alive:
+            continue
+        assert tuple(boxes[g, 1:4][::-1]) == r.origin and tuple(boxes[g, 4:7][::-1]) == r.dims
+        want = r.phi.astype(np.float32)
+        assert (np.abs(phi[g] - want) <= np.spacing(np.abs(want))).all()
