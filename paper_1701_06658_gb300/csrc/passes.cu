@@ -1010,13 +1010,13 @@ __device__ __forceinline__ void scan_line_regs(float* L, int n, int st, float pa
         if (j < n) L[j * st] = r[j];
 }
 
-// The scan of a periodic line of n magnitudes in shared memory: twice around
-// in each direction.
+// The scan of a periodic line of n values in shared memory (their magnitudes
+// go in and come out): twice around in each direction.
 __device__ __forceinline__ void scan_line_wrap(float* L, int n, int st) {
-    float f = L[0];
+    float f = fabsf(L[0]);
     for (int j = 1; j < 2 * n; ++j) {
         const int i = j < n ? j : j - n;
-        f = fminf(L[i * st], f + 1.0f);
+        f = fminf(fabsf(L[i * st]), f + 1.0f);
         L[i * st] = f;
     }
     for (int j = 2 * n - 2; j >= 0; --j) {
@@ -1052,6 +1052,12 @@ __device__ __forceinline__ void scan_seg_regs(float (&r)[L], int seg, float eps)
     for (int j = 0; j < kRedistReach; ++j) r[L - 1 - j] = fminf(r[L - 1 - j], cb + (float)(j + 1));
 }
 
+// Magnitude d with the sign of cell j of a segment whose positive cells are
+// the bits of m.
+__device__ __forceinline__ float with_sign(float d, unsigned m, int j) {
+    return __uint_as_float(__float_as_uint(d) | (~(m << (31 - j)) & 0x80000000u));
+}
+
 // Plane pass of the re-initialisation: a CTA of NT = 4 * SIDE threads takes
 // one (box, slab of kSlab planes) item at a time and walks its planes in z
 // order.  Planes of phi_c stream into a 3-slot shared-memory ring by bulk
@@ -1065,10 +1071,15 @@ __device__ __forceinline__ void scan_seg_regs(float (&r)[L], int seg, float eps)
 // cells of a segment at once, and only those load their neighbours' values
 // for the planar-exact distance; every other cell starts at eps.  The x scan
 // runs in the owner's registers (one carry exchange between the four lanes
-// of a row) and goes to the grid G; thread (c, s) then scans rows [s L, s L +
-// L) of column c the same way and stores plane z with the signs of phi_c put
-// back.  A full periodic axis takes a serial scan twice around the line by
-// one lane.  Every wait on a copy is bounded: on expiry the CTA records
+// of a row) and goes with the signs of phi_c to the grid G; thread (c, s) then
+// scans rows [s L, s L + L) of column c the same way and stores plane z.  A
+// full periodic axis takes a serial scan twice around the line by one lane.
+//
+// The pass is bound by its instructions, so what cannot change is left out:
+// a plane without a positive cell in itself and both neighbours is -eps (the
+// halo planes, about a quarter of a box), and the rows of a warp without a
+// reference cell stay +-eps, their scan skipped and, where they were -eps in
+// the plane before, not written again.  Every wait on a copy is bounded: on expiry the CTA records
 // LSGG_ERR_TIMEOUT, halts the step, drains its copies (bounded) and returns.
 constexpr int kRedistLanes = 4;      // lanes per row (x phase) and per column (y phase)
 __host__ __device__ constexpr size_t redist_layout_bytes(int side) {  // barriers, 3 plane slots, G, sign words, lists
@@ -1166,6 +1177,8 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
         request(z0);
         request(z0 + 1);
         unsigned fresh = 7u;                                // slots whose sign words are still to be made
+        unsigned anyp = 0u;                                 // bit k: slot k's plane has a positive cell
+        bool flat = false;                                  // this warp's rows of G are -eps throughout
         for (int z = z0; z < z1; ++z) {
             bool ok = true;
 #pragma unroll
@@ -1193,7 +1206,8 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
             const float* Pc = slots + kc * PA;
             const float* Pp = slots + kp * PA;
             // sign words of the planes that entered the ring: plane z + 1, and at
-            // the slab's start planes z - 1 and z as well
+            // the slab's start planes z - 1 and z as well; the barrier that
+            // publishes a plane's words tells whether it has a positive cell
             fresh |= 1u << kp;
 #pragma unroll
             for (int k = 0; k < 3; ++k)
@@ -1204,17 +1218,26 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
                     unsigned w = 0u;
 #pragma unroll
                     for (int j = 0; j < L; ++j) w |= (row[j] > 0.0f ? 1u : 0u) << j;
-                    W[k * WS + t] = r < ny ? w & valid : 0u;
+                    w = r < ny ? w & valid : 0u;
+                    W[k * WS + t] = w;
+                    anyp = __syncthreads_or(w != 0u) ? anyp | (1u << k) : anyp & ~(1u << k);
                 }
             fresh = 0u;
-            __syncthreads();
-            // classification and the x scan of row r, segment s
-            float rr[L];
+            float* const dst = B.Y + nb.off + (long long)z * ps;
+            if (anyp == 0u) {
+                // no positive cell in planes z - 1 .. z + 1: no reference cell,
+                // and every cell is -eps (the plane's padding included)
+                if (z + 1 < z1) request(z + 2);
+                for (int q = t; q < ps / 4; q += NT) reinterpret_cast<float4*>(dst)[q] = fill;
+                continue;
+            }
+            // classification and the x scan of row r, segment s; G takes the
+            // magnitudes with the signs of phi_c
             {
                 const unsigned* Wc = W + kc * WS;
+                const unsigned m0 = Wc[t];                          // 0 past ny
                 unsigned ref = 0u;
                 if (r < ny) {
-                    const unsigned m0 = Wc[t];
                     unsigned lbit, rbit;
                     if (s > 0) lbit = (Wc[t - 1] >> (L - 1)) & 1u;
                     else lbit = fx ? (Wc[r * LANES + sl] >> jl) & 1u : 0u;
@@ -1227,71 +1250,98 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
                     const unsigned mZm = W[km * WS + t], mZp = W[kp * WS + t];
                     ref = ((m0 ^ mL) | (m0 ^ mR) | (m0 ^ mU) | (m0 ^ mD) | (m0 ^ mZm) | (m0 ^ mZp)) & valid;
                 }
-                // the warp's reference cells into its list (lane order), then
-                // spread evenly over its lanes: planar-exact distance from the
-                // opposite-sign neighbours -> G
-                const int lane = t & 31;
-                const int cnt = __popc(ref);
-                int pre = cnt;
+                float* const grow = G + r * PG + x0;
+                if (__any_sync(0xffffffffu, ref != 0u)) {
+                    flat = false;
+                    // the warp's reference cells into its list (lane order), then
+                    // spread evenly over its lanes: planar-exact distance from the
+                    // opposite-sign neighbours -> G
+                    const int lane = t & 31;
+                    const int cnt = __popc(ref);
+                    int pre = cnt;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, pre, o);
-                    if (lane >= o) pre += v;
-                }
-                const int total = __shfl_sync(0xffffffffu, pre, 31);
-                pre -= cnt;
-                for (unsigned m = ref; m; m &= m - 1u) RL[pre++] = (unsigned short)((r << 8) | (x0 + __ffs(m) - 1));
-                __syncwarp();
-                for (int q = lane; q < total; q += 32) {
-                    const unsigned e = RL[q];
-                    const int ry = (int)(e >> 8), x = (int)(e & 0xffu);
-                    const int i = ry * nx + x;
-                    const float v = Pc[i];
-                    const bool pos = v > 0.0f;
-                    const float xl = x > 0 ? Pc[i - 1] : (fx ? Pc[i + nx - 1] : -eps);
-                    const float xr = x < nx - 1 ? Pc[i + 1] : (fx ? Pc[i - nx + 1] : -eps);
-                    const float yl = ry > 0 ? Pc[i - nx] : (fy ? Pc[i + n - nx] : -eps);
-                    const float yr = ry < ny - 1 ? Pc[i + nx] : (fy ? Pc[i - n + nx] : -eps);
-                    G[ry * PG + x] = ref_magnitude(fabsf(v), opp_max(pos, xl, xr), opp_max(pos, yl, yr),
-                                                   opp_max(pos, Pm[i], Pp[i]), eps);
-                }
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < L; ++j) {
-                    const float g = G[r * PG + x0 + j];            // in bounds; used at reference cells only
-                    rr[j] = (ref >> j) & 1u ? g : eps;
-                }
-                if (!fx) scan_seg_regs<L, LANES>(rr, s, eps);
-                // rows past ny and cells past nx of G are written but never read
-#pragma unroll
-                for (int j = 0; j < L; ++j) G[r * PG + x0 + j] = rr[j];
-                if (fx) {                                   // periodic x: the row twice around, one lane
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+                        if (lane >= o) pre += v;
+                    }
+                    const int total = __shfl_sync(0xffffffffu, pre, 31);
+                    pre -= cnt;
+                    for (unsigned m = ref; m; m &= m - 1u) RL[pre++] = (unsigned short)((r << 8) | (x0 + __ffs(m) - 1));
                     __syncwarp();
-                    if (s == 0 && r < ny) scan_line_wrap(G + r * PG, nx, 1);
+                    for (int q = lane; q < total; q += 32) {
+                        const unsigned e = RL[q];
+                        const int ry = (int)(e >> 8), x = (int)(e & 0xffu);
+                        const int i = ry * nx + x;
+                        const float v = Pc[i];
+                        const bool pos = v > 0.0f;
+                        const float xl = x > 0 ? Pc[i - 1] : (fx ? Pc[i + nx - 1] : -eps);
+                        const float xr = x < nx - 1 ? Pc[i + 1] : (fx ? Pc[i - nx + 1] : -eps);
+                        const float yl = ry > 0 ? Pc[i - nx] : (fy ? Pc[i + n - nx] : -eps);
+                        const float yr = ry < ny - 1 ? Pc[i + nx] : (fy ? Pc[i - n + nx] : -eps);
+                        G[ry * PG + x] = ref_magnitude(fabsf(v), opp_max(pos, xl, xr), opp_max(pos, yl, yr),
+                                                       opp_max(pos, Pm[i], Pp[i]), eps);
+                    }
+                    __syncwarp();
+                    float rr[L];
+#pragma unroll
+                    for (int j = 0; j < L; ++j) {
+                        const float g = grow[j];                   // in bounds; used at reference cells only
+                        rr[j] = (ref >> j) & 1u ? g : eps;
+                    }
+                    if (!fx) scan_seg_regs<L, LANES>(rr, s, eps);
+                    else {                                  // periodic x: the row twice around, one lane
+#pragma unroll
+                        for (int j = 0; j < L; ++j) grow[j] = rr[j];
+                        __syncwarp();
+                        if (s == 0 && r < ny) scan_line_wrap(G + r * PG, nx, 1);
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < L; ++j) rr[j] = grow[j];
+                    }
+                    // rows past ny and cells past nx of G are written but never used
+#pragma unroll
+                    for (int j = 0; j < L; ++j) grow[j] = with_sign(rr[j], m0, j);
+                } else if (!__all_sync(0xffffffffu, m0 == 0u)) {
+                    // no reference cell in the warp's rows: +-eps
+                    flat = false;
+#pragma unroll
+                    for (int j = 0; j < L; ++j) grow[j] = with_sign(eps, m0, j);
+                } else if (!flat) {
+                    flat = !fy;                             // the periodic y scan writes to G
+#pragma unroll
+                    for (int j = 0; j < L; ++j) grow[j] = -eps;
                 }
             }
             __syncthreads();                                // G holds the x scans; the slot of z - 1 is free
             if (z + 1 < z1) request(z + 2);
-            // y scan of column c = r, rows [s L, s L + L), then the signs of plane z back
+            // y scan of column c = r, rows [s L, s L + L) with the signs kept
             {
                 const int c = r;
-                if (fy) {                                   // periodic y: the column twice around, one lane
+                const float* const gcol = G + x0 * PG + c;
+                float* dc = dst + x0 * nx + c;
+                const int nrow = c < nx ? min(ny - x0, L) : 0;         // rows of the segment to store
+                float rr[L];
+                if (!fy) {
+                    float sg[L];
+#pragma unroll
+                    for (int j = 0; j < L; ++j) {
+                        sg[j] = gcol[j * PG];                          // in bounds; rows past ny are eps
+                        rr[j] = fabsf(sg[j]);
+                    }
+                    scan_seg_regs<L, LANES>(rr, s, eps);
+#pragma unroll
+                    for (int j = 0; j < L; ++j) {
+                        if (j < nrow) *dc = copysignf(rr[j], sg[j]);
+                        dc += nx;
+                    }
+                } else {                                    // periodic y: the column twice around, one lane
                     if (s == 0 && c < nx) scan_line_wrap(G + c, ny, PG);
                     __syncwarp();
-                }
 #pragma unroll
-                for (int j = 0; j < L; ++j) {
-                    const float g = G[(x0 + j) * PG + c];          // in bounds; rows past ny are eps
-                    rr[j] = x0 + j < ny ? g : eps;
-                }
-                if (!fy) scan_seg_regs<L, LANES>(rr, s, eps);
-                float* dst = B.Y + nb.off + (long long)z * ps + c;
-                const float* pcol = Pc + c;
-#pragma unroll
-                for (int j = 0; j < L; ++j) {
-                    const int y = x0 + j;
-                    const float sgn = pcol[min(y, ny - 1) * nx];   // in bounds; stored only inside the plane
-                    if (c < nx && y < ny) dst[y * nx] = sgn > 0.0f ? rr[j] : -rr[j];
+                    for (int j = 0; j < L; ++j) {
+                        if (j < nrow) *dc = Pc[(x0 + j) * nx + c] > 0.0f ? fabsf(gcol[j * PG]) : -fabsf(gcol[j * PG]);
+                        dc += nx;
+                    }
                 }
             }
         }
