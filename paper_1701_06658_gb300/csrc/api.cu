@@ -590,6 +590,7 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     c->B.bf16 = cfg_in->storage == LSGG_STORAGE_BF16 ? 1 : 0;
     c->B.redist = cfg_in->redist;
     c->B.wait_limit = kWaitIters;
+    c->B.tile_x = cfg_in->physics != LSGG_PHYSICS_IDEAL && ncell > kWideTileCells ? 32 : 16;
     if (configure_step_kernels(c->B) != cudaSuccess) return bail(CUDA_FAIL());
     if (c->B.bf16)
         for (int k = 0; k < kNumClasses; ++k)

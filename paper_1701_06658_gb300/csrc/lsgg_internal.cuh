@@ -37,7 +37,9 @@ constexpr int kTiers = 5;               // pass path: boxes with x, y sides <= 3
 constexpr int kPassChunk = 256;         // columns per column item of the pass path
 constexpr int kSlab = 8;                // planes per slab item of the pass path (default; autotuned)
 constexpr int kMinSlab = 4;             // the smallest slab the autotuner tries (sizes the slab item list)
-constexpr int kTileX = 8, kTileY = 32, kTileZ = 8;    // domain tiles of the field pass
+constexpr int kTileThreads = 256;       // columns of a field-pass tile, one per thread
+constexpr int kTileZ = 8;               // planes of a field-pass tile (its columns: StepBuffers::tile_x)
+constexpr long long kWideTileCells = 96LL << 20;   // domains above this with physics: 32-column tiles
 constexpr int kTileCap = 128;           // boxes listed per tile (more: the tile scans all boxes)
 
 struct Box {
@@ -216,7 +218,8 @@ struct StepBuffers {
     int pocc[kTiers][5];            // resident CTAs per SM of those kernels (the grids' upper bound)
     int slab;                       // planes per slab item of p_redist_xy (kSlab unless autotuned)
     long long* bu_part;             // box update: per chunk of kBuChunk boxes kBuVals sums, then their bases
-    // field pass: boxes overlapping each domain tile of kTileX x kTileY x kTileZ cells
+    // field pass: boxes overlapping each domain tile of tile_x x (256 / tile_x) x kTileZ cells
+    int tile_x;                     // 16, or 32 (set at creation; the lists are sized for it)
     int* tile_cnt;                  // [n_tiles]
     int* tile_list;                 // [n_tiles * kTileCap]
     int ntile[3];

@@ -35,12 +35,16 @@
 // use.
 #include <cfloat>
 #include <climits>
+#include <type_traits>
 
 #include "bulk_copy.cuh"
 #include "group.cuh"
 #include "kernels_common.cuh"
 
 namespace lsgg {
+
+using Yes = std::true_type;
+using No = std::false_type;
 
 constexpr int kZB = 8;               // planes loaded ahead by the column passes
 constexpr int kReachP = kRedistReach;
@@ -690,8 +694,8 @@ k_bin(StepBuffers B1, GroupRef grp) {
             B.bounds[b] = bd;
         }
         int ts[3], tc[3];
-        axis_tiles(bx.ox, bx.nx, D.nx, kTileX, B.ntile[0], ts[0], tc[0]);
-        axis_tiles(bx.oy, bx.ny, D.ny, kTileY, B.ntile[1], ts[1], tc[1]);
+        axis_tiles(bx.ox, bx.nx, D.nx, B.tile_x, B.ntile[0], ts[0], tc[0]);
+        axis_tiles(bx.oy, bx.ny, D.ny, kTileThreads / B.tile_x, B.ntile[1], ts[1], tc[1]);
         axis_tiles(bx.oz, bx.nz, D.nz, kTileZ, B.ntile[2], ts[2], tc[2]);
         const int n = tc[0] * tc[1] * tc[2];
         for (int k = lane; k < n; k += 32) {
@@ -725,15 +729,33 @@ k_clear_tiles_group(GroupRef grp) {
 // largest values per cell (where wanted with their grains) in registers,
 // ordered by phi_p and, at equal phi_p, by the smaller grain id first -- the
 // order of the box-streaming kernels' 64-bit keys (phi_p, -id) under
-// atomicMax, so m and the ID-field are identical.  Per listed box the CTA first stages, in shared
-// memory, how the tile maps into the box: on an axis where the box's cells
-// in the tile keep one box-local offset (all but boxes spanning nearly the
-// whole domain), the mask of the tile's rows / columns / planes it covers
-// and one arena offset for the tile's corner, so that the per-thread work is
-// a mask test per column and an add per cell; other boxes take the general
-// cyclic path.
-// CTAs per SM the value-only field pass is sized for.
-constexpr int kFieldBlocks = 5;
+// atomicMax, so m and the ID-field are identical.  Per listed box the CTA
+// first stages, in shared memory, how the tile maps into the box: on an axis
+// where the box's cells in the tile keep one box-local offset (all but boxes
+// spanning nearly the whole domain), the mask of the tile's rows / columns /
+// planes it covers and one arena offset for the tile's corner, so that the
+// per-thread work is a mask test per column and an add per cell; other boxes
+// take the general cyclic path.
+//
+// Tile shape.  A box row in a tile is a short unaligned run of its arena, so
+// each row costs about one 32-byte sector more than its cells; wider tiles
+// waste fewer sectors and more lanes (a box 30 cells wide covers half of a
+// 32-wide tile's lanes, four fifths of an 8-wide one's).  16 x 16 is the
+// better of the two sides at most sizes: GB300, field pass alone, 8 x 32 /
+// 16 x 16 / 32 x 8: ideal 256^3 0.46 / 0.41 / 0.50 ms, magnetic 384^3 2.94 /
+// 2.33 / 2.46.  With the ID-field at 512^3 the partly written sectors of two
+// output arenas leave L2 before the neighbour tile completes them (30 GB of
+// DRAM reads for 4 GB of phi_p at 8 x 32): 11.1 / 8.3 / 6.9 ms, and 6.4 with
+// the first kFieldSlots columns of a thread kept in shared memory for the
+// second sweep, so domains of more than kWideTileCells cells with physics
+// take 32 x 8 and the slots.  With the second sweep on grains decoded once and
+// whole-tile columns apart from partial ones: 0.38 / 2.07 / 5.7 ms (ideal 256^3,
+// magnetic 384^3, Read-Shockley 512^3).  Three CTAs per SM with grains: four
+// thrash L2 (16 x 16, magnetic 384^3: 3.4 ms).
+
+constexpr int kFieldSlots = 8;
+__host__ __device__ constexpr int field_slots(int tx) { return tx == 32 ? kFieldSlots : 0; }
+constexpr size_t field_smem(int tx) { return sizeof(float) * kTileThreads * kTileZ * field_slots(tx); }
 
 struct TileBox {
     long long off;            // affine: arena offset of tile cell (0, 0, 0); general: of the box
@@ -798,13 +820,20 @@ __device__ __forceinline__ void stage_tile_box(const StepBuffers& B, int b, int 
     t.zm = m;
 }
 
-// (v, id) enters the top two (v1, i1) >= (v2, i2) of a cell; boxes come in
-// ascending grain id, so an equal value never displaces an earlier one (the
-// lowest id on ties).  Absent entries are (-inf, -1).
-__device__ __forceinline__ void top2_insert(float v, int id, float& v1, int& i1, float& v2, int& i2) {
-    const bool c1 = v > v1, c2 = v > v2;
-    i2 = c1 ? i1 : (c2 ? id : i2);
-    i1 = c1 ? id : i1;
+// The value v of list entry k enters the top two of cell zz of a column: the
+// values v1 >= v2, the entries as bytes of p1, p2 (four cells a word; kk is k in
+// every byte).  Boxes come in ascending grain id, so an equal value never
+// displaces an earlier one (the lowest id on ties).
+constexpr unsigned kOldFirst = 0xffu, kOldSecond = 0xfeu;   // entries of the batches before this one, or none
+static_assert(kTileCap <= 0xfe, "a list entry is a byte beside the two marks");
+__device__ __forceinline__ unsigned byte_of(unsigned p, int b) { return __byte_perm(p, 0u, 0x4440u | b); }
+__device__ __forceinline__ void top2_insert(float v, unsigned kk, float& v1, float& v2, unsigned& p1, unsigned& p2,
+                                            int b) {
+    const unsigned sel = 0x3210u + ((4u) << (4 * b));       // byte b from the second word
+    const bool c1 = v > v1, c2 = v > v2;                    // c1 implies c2
+    const unsigned from = c1 ? p1 : kk;
+    if (c2) p2 = __byte_perm(p2, from, sel);
+    if (c1) p1 = __byte_perm(p1, kk, sel);
     v2 = fmaxf(v2, fminf(v1, v));
     v1 = fmaxf(v1, v);
 }
@@ -820,81 +849,143 @@ __device__ __forceinline__ void top2_values(float v, float& v1, float& v2) {
 // suffice: a box cell whose phi_p equals the largest value is either its
 // holder, whose m is the second value, or ties with it, and then the two
 // values are equal; every other cell's m is the largest value.  The insertion
-// is then three instructions a cell instead of twelve and the top two take 16
-// registers instead of 32.  The pass is bound by the latency of its column
-// loads (each warp load touches four rows of eight cells, about two 32-byte
-// sectors a row): the freed registers go into a fifth CTA per SM.  Measured on
-// GB300, 256^3 / 5000 grains, whole step: 2.33 ms with the grains tracked at
-// four CTAs, 2.26 / 2.23 / 2.42 ms values only at four / five / six CTAs (six
-// spills).
-template <bool IDS, bool IDF, bool DBG, bool GRP>
-__global__ void __launch_bounds__(kTileX * kTileY, IDS ? 3 : (GRP ? 4 : kFieldBlocks))
+// is then three instructions a cell instead of eight.  Measured on GB300,
+// 256^3 / 5000 grains, whole step: 2.33 ms with the grains tracked, 2.23
+// without.
+template <int TX, bool IDS, bool IDF, bool DBG, bool GRP>
+__global__ void __launch_bounds__(kTileThreads, IDS ? 3 : (GRP ? 4 : 5))
 p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
     static_assert(!(GRP && (IDF || DBG)), "step groups run ideal growth without intermediates");
     static_assert(IDS || !(IDF || DBG), "the ID-field and the intermediates need the top two's grains");
+    constexpr int TY = kTileThreads / TX;
+    constexpr int SLOTS = field_slots(TX);
+    static_assert(TX <= 32 && TY <= 32, "a tile's columns and rows are bits of a word");
+    constexpr bool MID = IDF || DBG;
     __shared__ TileBox s_tb[kTileCap];
-    __shared__ int s_id[IDS ? kTileCap : 1];
+    __shared__ int s_id[IDS ? 256 : 1];             // grain of each list entry in ascending order; none: -1
+    __shared__ int s_in[IDS ? kTileCap : 1];        // the list as binned
     __shared__ int s_gb[GRP ? kMaxGroup + 1 : 1];
+    extern __shared__ float s_val[];                // SLOTS x kTileZ x kTileThreads
     if (!GRP && halted(B1)) return;
+    if (IDS && threadIdx.x >= kTileCap && threadIdx.x < 256) s_id[threadIdx.x] = -1;
     const int n_all = GRP ? group_scan(grp, kItemTiles, 0, true, s_gb) : B1.n_tiles;
-    const int lx = threadIdx.x % kTileX, ly = threadIdx.x / kTileX;
+    const int lx = threadIdx.x % TX, ly = threadIdx.x / TX;
     for (int gtile = blockIdx.x; gtile < n_all; gtile += gridDim.x) {
         int tile;
         const StepBuffers& B = member<GRP>(B1, grp, s_gb, gtile, tile);
         const Domain D = B.dom;
         const float eps = D.eps;
-        const float* const Y = B.Y;
         const int ntx = B.ntile[0], nty = B.ntile[1];
         const int tx = tile % ntx, tyz = tile / ntx, ty = tyz % nty, tz = tyz / nty;
-        const int tx0 = tx * kTileX, ty0 = ty * kTileY, z0 = tz * kTileZ;
+        const int tx0 = tx * TX, ty0 = ty * TY, z0 = tz * kTileZ;
         const int x = tx0 + lx, y = ty0 + ly;
         const bool col = x < D.nx && y < D.ny;
-        const int ext_x = min(kTileX, D.nx - tx0), ext_y = min(kTileY, D.ny - ty0);
+        const int ext_x = min(TX, D.nx - tx0), ext_y = min(TY, D.ny - ty0);
         const int nzt = min(kTileZ, D.nz - z0);
         const int cnt = B.tile_cnt[tile];
         const bool all = cnt > kTileCap;            // list overflowed: test every box in batches
         const int n_total = all ? B.n_boxes : cnt;
+        const bool multi = n_total > kTileCap;      // several batches: their cells' keys stay in T between them
+        ulonglong2* const T2 = reinterpret_cast<ulonglong2*>(B.T);
+        auto tcell = [&](int zz) { return ((long long)(z0 + zz) * D.ny + y) * D.nx + x; };
         float v1[kTileZ], v2[kTileZ];
-        int i1[IDS ? kTileZ : 1], i2[IDS ? kTileZ : 1];
+        unsigned p1[IDS ? kTileZ / 4 : 1], p2[IDS ? kTileZ / 4 : 1];
+        int id1[MID ? kTileZ : 1], id2[MID ? kTileZ : 1];
+        auto reset_entries = [&]() {
 #pragma unroll
-        for (int zz = 0; zz < kTileZ; ++zz) {
-            v1[zz] = v2[zz] = -INFINITY;
-            if (IDS) i1[zz] = i2[zz] = -1;
-        }
-        // two sweeps over the tile's boxes: 0 builds the top two, 1 writes phi_c
+            for (int h = 0; h < (IDS ? kTileZ / 4 : 0); ++h) {
+                p1[h] = 0x01010101u * kOldFirst;
+                p2[h] = 0x01010101u * kOldSecond;
+            }
+        };
 #pragma unroll
-        for (int sweep = 0; sweep < 2; ++sweep) {
-            if (sweep == 1) {
-                ulonglong2* T2 = reinterpret_cast<ulonglong2*>(B.T);
-                const bool keep = IDS && B.keep_field != 0;
+        for (int zz = 0; zz < kTileZ; ++zz) v1[zz] = v2[zz] = -INFINITY;
+        reset_entries();
+        int slot;                                   // this thread's next slot of s_val
+        // One box's column (list entry k, arena offset oc of the tile's plane
+        // 0, planes zm) in sweep SW; FULL: every plane of the tile; GEN: a box
+        // in general position (its planes wrap).
+        auto column = [&](auto sw, auto full, auto gen, const TileBox& t, int k, long long oc, unsigned zm) {
+            constexpr int SW = decltype(sw)::value;
+            constexpr bool FULL = decltype(full)::value, GEN = decltype(gen)::value;
+            const unsigned ps = (unsigned)t.ps;
+            const int dz = GEN ? t.dz : 0;
+            auto at = [&](int zz) {                 // offset of the column's cell zz
+                if (!GEN) return (unsigned)zz * ps;
+                const int lz = dz + zz;
+                return (unsigned)(lz >= D.nz ? lz - D.nz : lz) * ps;
+            };
+            const float* const yc = B.Y + oc;
+            float* const keep = s_val + slot * (kTileZ * kTileThreads) + threadIdx.x;
+            float v[kTileZ];
+            if (SW == 1 && SLOTS > 0 && slot < SLOTS) {
+#pragma unroll
+                for (int zz = 0; zz < kTileZ; ++zz) v[zz] = keep[zz * kTileThreads];
+            } else {
+#pragma unroll
+                for (int zz = 0; zz < kTileZ; ++zz)
+                    v[zz] = FULL || ((zm >> zz) & 1u) ? __ldg(yc + at(zz)) : -INFINITY;
+            }
+            if (SW == 0) {
+                if (SLOTS > 0 && slot < SLOTS) {
+#pragma unroll
+                    for (int zz = 0; zz < kTileZ; ++zz) keep[zz * kTileThreads] = v[zz];
+                }
 #pragma unroll
                 for (int zz = 0; zz < kTileZ; ++zz) {
-                    if (IDS && keep && col && zz < nzt)
-                        T2[((long long)(z0 + zz) * D.ny + y) * D.nx + x] =
-                            make_ulonglong2(i1[zz] >= 0 ? make_key(v1[zz], i1[zz]) : 0ull,
-                                            i2[zz] >= 0 ? make_key(v2[zz], i2[zz]) : 0ull);
-                    // as m: absent is -eps, -0 becomes +0
-                    v1[zz] = v1[zz] > -INFINITY ? v1[zz] + 0.0f : -eps;
-                    v2[zz] = v2[zz] > -INFINITY ? v2[zz] + 0.0f : -eps;
+                    if constexpr (IDS)
+                        top2_insert(v[zz], 0x01010101u * (unsigned)k, v1[zz], v2[zz], p1[zz / 4], p2[zz / 4], zz % 4);
+                    else top2_values(v[zz], v1[zz], v2[zz]);
+                }
+            } else {
+                float* const zc = B.Z + oc;
+                int* const ic = IDF ? B.IDF + oc : nullptr;
+#pragma unroll
+                for (int zz = 0; zz < kTileZ; ++zz) {
+                    if (!FULL && !((zm >> zz) & 1u)) continue;
+                    const unsigned o = at(zz);
+                    bool top;
+                    if constexpr (MID) top = id1[zz] == t.id;
+                    else top = v[zz] == v1[zz];
+                    const float m = top ? v2[zz] : v1[zz];
+                    const float pc = 0.5f * (v[zz] - m);
+                    zc[o] = pc;
+                    if constexpr (MID) {
+                        const int mid = top ? id2[zz] : id1[zz];
+                        if constexpr (IDF) ic[o] = mid;
+                        if constexpr (DBG) {
+                            dbg.m[oc + o] = m;
+                            dbg.idm[oc + o] = mid;
+                            dbg.phic[oc + o] = pc;
+                            dbg.phip[oc + o] = v[zz];
+                        }
+                    }
                 }
             }
+            if (SLOTS > 0) ++slot;
+        };
+        // a sweep over the tile's boxes: 0 builds the top two, 1 writes phi_c
+        auto sweep = [&](auto sw) {
+            constexpr int SW = decltype(sw)::value;
+            slot = multi ? SLOTS : 0;
             for (int base = 0; base < n_total; base += kTileCap) {
                 const int nb = min(kTileCap, n_total - base);
                 // one batch (the tile's whole list): the first sweep's staging serves both
-                if (sweep == 0 || n_total > kTileCap) {
+                if (SW == 0 || multi) {
                     __syncthreads();                // previous batch done with s_tb
                     if constexpr (IDS) {            // in ascending id: each box's rank in the list
-                        for (int k = threadIdx.x; k < nb; k += blockDim.x)
-                            s_id[k] = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
+                        for (int k = threadIdx.x; k < nb; k += kTileThreads)
+                            s_in[k] = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
                         __syncthreads();
-                        for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-                            const int b = s_id[k];
+                        for (int k = threadIdx.x; k < nb; k += kTileThreads) {
+                            const int b = s_in[k];
                             int rank = 0;
-                            for (int q = 0; q < nb; ++q) rank += s_id[q] < b;
+                            for (int q = 0; q < nb; ++q) rank += s_in[q] < b;
+                            s_id[rank] = b;
                             stage_tile_box(B, b, tx0, ty0, z0, ext_x, ext_y, nzt, s_tb[rank]);
                         }
                     } else {
-                        for (int k = threadIdx.x; k < nb; k += blockDim.x) {
+                        for (int k = threadIdx.x; k < nb; k += kTileThreads) {
                             const int b = all ? base + k : B.tile_list[(long long)tile * kTileCap + k];
                             stage_tile_box(B, b, tx0, ty0, z0, ext_x, ext_y, nzt, s_tb[k]);
                         }
@@ -906,70 +997,81 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
                     const TileBox& t = s_tb[k];
                     const unsigned zaff = t.zm;
                     const unsigned zm = zaff & 0xffu;
-                    const int id = t.id, ps = t.ps;
-                    // the column's cells at arena offsets oc + lz(zz) * ps
-                    auto cells = [&](const long long oc, auto lz) {
-                        const float* yc = Y + oc;
-                        float v[kTileZ];
-                        if (zm == 0xffu) {              // the whole column (uniform)
-#pragma unroll
-                            for (int zz = 0; zz < kTileZ; ++zz) v[zz] = __ldg(yc + (size_t)(lz(zz) * (unsigned)ps));
-                        } else {
-#pragma unroll
-                            for (int zz = 0; zz < kTileZ; ++zz)
-                                v[zz] = (zm >> zz) & 1u ? __ldg(yc + (size_t)(lz(zz) * (unsigned)ps)) : -INFINITY;
-                        }
-                        if (sweep == 0) {
-#pragma unroll
-                            for (int zz = 0; zz < kTileZ; ++zz) {
-                                if constexpr (IDS) top2_insert(v[zz], id, v1[zz], i1[zz], v2[zz], i2[zz]);
-                                else top2_values(v[zz], v1[zz], v2[zz]);
-                            }
-                        } else {
-                            float* zc = B.Z + oc;
-#pragma unroll
-                            for (int zz = 0; zz < kTileZ; ++zz) {
-                                if (!((zm >> zz) & 1u)) continue;
-                                const size_t o = lz(zz) * (unsigned)ps;
-                                bool top;
-                                if constexpr (IDS) top = i1[zz] == id;
-                                else top = v[zz] == v1[zz];
-                                const float m = top ? v2[zz] : v1[zz];
-                                const float pc = 0.5f * (v[zz] - m);
-                                zc[o] = pc;
-                                if constexpr (IDF || DBG) {
-                                    int mid = top ? i2[zz] : i1[zz];
-                                    if (!(m > -eps)) mid = -1;
-                                    if (IDF) B.IDF[oc + o] = mid;
-                                    if (DBG) {
-                                        dbg.m[oc + o] = m;
-                                        dbg.idm[oc + o] = mid;
-                                        dbg.phic[oc + o] = pc;
-                                        dbg.phip[oc + o] = v[zz];
-                                    }
-                                }
-                            }
-                        }
-                    };
                     if (zaff >> 31) {                   // affine (uniform across the CTA)
                         if (!((t.xmask >> lx) & (t.ymask >> ly) & 1u)) continue;
-                        cells(t.off + (long long)(ly * t.nx + lx), [](int zz) { return zz; });
+                        const long long oc = t.off + (long long)(ly * t.nx + lx);
+                        if (zm == 0xffu) column(sw, Yes{}, No{}, t, k, oc, zm);
+                        else column(sw, No{}, No{}, t, k, oc, zm);
                     } else {
                         if (!zm) continue;
                         int bxl = t.dx + lx, byl = t.dy + ly;
                         if (bxl >= D.nx) bxl -= D.nx;
                         if (byl >= D.ny) byl -= D.ny;
                         if (bxl >= t.nx || byl >= t.ny) continue;
-                        const int dz = t.dz, dnz = D.nz;
-                        cells(t.off + (long long)byl * t.nx + bxl, [dz, dnz](int zz) {
-                            const int lz = dz + zz;
-                            return lz >= dnz ? lz - dnz : lz;
-                        });
+                        column(sw, No{}, Yes{}, t, k, t.off + (long long)byl * t.nx + bxl, zm);
+                    }
+                }
+                if constexpr (IDS && SW == 0) {
+                    // the batch's entries as grains, merged with the earlier batches' in T
+                    if (multi) {
+#pragma unroll
+                        for (int zz = 0; zz < kTileZ; ++zz) {
+                            if (zz >= nzt) continue;
+                            int o1 = -1, o2 = -1;
+                            if (base > 0) {
+                                const ulonglong2 key = T2[tcell(zz)];
+                                o1 = key_id(key.x);
+                                o2 = key_id(key.y);
+                            }
+                            auto grain = [&](unsigned e) {
+                                return e == kOldFirst ? o1 : (e == kOldSecond ? o2 : s_id[e]);
+                            };
+                            const int i1 = grain(byte_of(p1[zz / 4], zz % 4)), i2 = grain(byte_of(p2[zz / 4], zz % 4));
+                            T2[tcell(zz)] = make_ulonglong2(i1 >= 0 ? make_key(v1[zz], i1) : 0ull,
+                                                            i2 >= 0 ? make_key(v2[zz], i2) : 0ull);
+                        }
+                        reset_entries();
                     }
                 }
             }
+        };
+        sweep(std::integral_constant<int, 0>{});
+        // the top two as the second sweep reads them: absent is -eps, -0 becomes
+        // +0; grains only of values above -eps (the others are no neighbours)
+#pragma unroll
+        for (int zz = 0; zz < kTileZ; ++zz) {
+            if constexpr (IDS) {
+                int i1 = s_id[byte_of(p1[zz / 4], zz % 4)], i2 = s_id[byte_of(p2[zz / 4], zz % 4)];
+                if (col && zz < nzt) {
+                    if (multi) {
+                        const ulonglong2 key = T2[tcell(zz)];
+                        i1 = key_id(key.x);
+                        i2 = key_id(key.y);
+                    } else if (B.keep_field) {
+                        T2[tcell(zz)] = make_ulonglong2(i1 >= 0 ? make_key(v1[zz], i1) : 0ull,
+                                                        i2 >= 0 ? make_key(v2[zz], i2) : 0ull);
+                    }
+                }
+                if constexpr (MID) {
+                    id1[zz] = v1[zz] > -eps ? i1 : -1;
+                    id2[zz] = v2[zz] > -eps ? i2 : -1;
+                }
+            }
+            v1[zz] = v1[zz] > -INFINITY ? v1[zz] + 0.0f : -eps;
+            v2[zz] = v2[zz] > -INFINITY ? v2[zz] + 0.0f : -eps;
         }
+        sweep(std::integral_constant<int, 1>{});
     }
+}
+
+// The field pass with the IDs or without, the intermediates of a debug step,
+// on a tile of `tx` columns.
+using FieldFn = void (*)(StepBuffers, GroupRef, PhysicsDev, DebugOut);
+static FieldFn field_fn(int tx, bool ids, bool idf, bool dg) {
+    if (tx == 32) return dg ? p_field<32, true, true, true, false> : p_field<32, true, true, false, false>;
+    if (idf) return dg ? p_field<16, true, true, true, false> : p_field<16, true, true, false, false>;
+    if (dg) return p_field<16, true, false, true, false>;
+    return ids ? p_field<16, true, false, false, false> : p_field<16, false, false, false, false>;
 }
 
 // ---------------------------------------------------------------------------
@@ -2111,16 +2213,21 @@ cudaError_t configure_passes(StepBuffers& B) {
             B.pgrid[t][k] = B.n_sm * B.pocc[t][k];
         }
     }
-    int of = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, false, false>, kTileX * kTileY, 0);
-    if (e != cudaSuccess) return e;
-    B.field_grid[0] = B.n_sm * (of < 1 ? 1 : of);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<true, true, false, false>, kTileX * kTileY, 0);
-    if (e != cudaSuccess) return e;
-    B.field_grid[1] = B.n_sm * (of < 1 ? 1 : of);
+    if (B.tile_x != 32) B.tile_x = 16;
+    for (int ids = 0; ids < 2; ++ids) {
+        int of = 0;
+        const void* f = reinterpret_cast<const void*>(field_fn(B.tile_x, ids, ids && B.tile_x == 32, false));
+        e = allow_max_dynamic_smem(f);
+        if (e == cudaSuccess && B.tile_x == 32)
+            e = allow_max_dynamic_smem(reinterpret_cast<const void*>(field_fn(32, true, true, true)));
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, f, kTileThreads, field_smem(B.tile_x));
+        if (e != cudaSuccess) return e;
+        B.field_grid[ids] = B.n_sm * (of < 1 ? 1 : of);
+    }
     B.bin_grid = B.n_sm;
     if (B.slab < kMinSlab) B.slab = kSlab;
-    const int tsz[3] = {kTileX, kTileY, kTileZ};
+    const int tsz[3] = {B.tile_x, kTileThreads / B.tile_x, kTileZ};
     const int dn[3] = {B.dom.nx, B.dom.ny, B.dom.nz};
     for (int a = 0; a < 3; ++a) B.ntile[a] = (dn[a] + tsz[a] - 1) / tsz[a];
     B.n_tiles = B.ntile[0] * B.ntile[1] * B.ntile[2];
@@ -2177,11 +2284,8 @@ cudaError_t launch_bin(const StepBuffers& B, cudaStream_t s) {
 cudaError_t launch_field(const StepBuffers& B, const PhysicsDev& phys, const DebugOut& dbg, cudaStream_t s) {
     const bool idf = phys.kind != LSGG_PHYSICS_IDEAL, dg = dbg.m != nullptr;
     const bool ids = idf || dg || B.keep_field;
-    auto k = idf   ? (dg ? p_field<true, true, true, false> : p_field<true, true, false, false>)
-             : dg  ? p_field<true, false, true, false>
-             : ids ? p_field<true, false, false, false>
-                   : p_field<false, false, false, false>;
-    k<<<B.field_grid[ids ? 1 : 0], kTileX * kTileY, 0, s>>>(B, GroupRef{nullptr, 0}, phys, dbg);
+    field_fn(B.tile_x, ids, idf, dg)<<<B.field_grid[ids ? 1 : 0], kTileThreads, field_smem(B.tile_x), s>>>(
+        B, GroupRef{nullptr, 0}, phys, dbg);
     return cudaGetLastError();
 }
 
@@ -2250,10 +2354,10 @@ cudaError_t configure_group_kernels(int n_sm) {
         for (int k = 0; k < 5; ++k) sh.pgrid[t][k] = n_sm * (o[k] < 1 ? 1 : o[k]);
     }
     int of = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<false, false, false, true>, kTileX * kTileY, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<16, false, false, false, true>, kTileThreads, 0);
     if (e != cudaSuccess) return e;
     sh.field[0] = n_sm * (of < 1 ? 1 : of);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<true, false, false, true>, kTileX * kTileY, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&of, p_field<16, true, false, false, true>, kTileThreads, 0);
     if (e != cudaSuccess) return e;
     sh.field[1] = n_sm * (of < 1 ? 1 : of);
     sh.bin = n_sm;
@@ -2271,8 +2375,8 @@ cudaError_t launch_bin_group(const StepBuffers& B0, const GroupRef& grp, cudaStr
 
 // ids: a member stores the field (lsgg_keep_field)
 cudaError_t launch_field_group(const StepBuffers& B0, const GroupRef& grp, bool ids, cudaStream_t s) {
-    auto k = ids ? p_field<true, false, false, true> : p_field<false, false, false, true>;
-    k<<<g_group_shapes.field[ids ? 1 : 0], kTileX * kTileY, 0, s>>>(B0, grp, PhysicsDev{}, DebugOut{});
+    auto k = ids ? p_field<16, true, false, false, true> : p_field<16, false, false, false, true>;
+    k<<<g_group_shapes.field[ids ? 1 : 0], kTileThreads, 0, s>>>(B0, grp, PhysicsDev{}, DebugOut{});
     return cudaGetLastError();
 }
 

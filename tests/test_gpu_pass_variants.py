@@ -91,3 +91,49 @@ def test_start_from_seeds_against_the_oracle(L, dims, G, big):
         assert tuple(boxes[g, 1:4][::-1]) == r.origin and tuple(boxes[g, 4:7][::-1]) == r.dims
         want = r.phi.astype(np.float32)
         assert (np.abs(phi[g] - want) <= np.spacing(np.abs(want))).all()
+
+
+def test_field_pass_with_overflowing_tile_lists(L):
+    """More boxes on a tile than its list holds: the tile takes every box in batches.  The ID-field is the
+    oracle's argmax of the step's own phi_p, m its value (copies of FP32 numbers: equal)."""
+    from oracle import lsgg_oracle as O
+    dims, G = (20, 22, 24), 300
+    quats = I.random_quaternions(8, G)
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(8, G, dims), quats=quats,
+                          physics=L.PHYSICS_READ_SHOCKLEY) as ms:
+        boxes, (phip, m, idm, phic, _) = ms.debug_step(1.0)
+    grains, pp = [], {}
+    for g in range(G):
+        if g not in phip:
+            grains.append(O.Grain(g, (0, 0, 0), np.full((1, 1, 1), -7.0), alive=False))
+            continue
+        b = boxes[g]
+        pp[g] = phip[g].astype(np.float64)
+        grains.append(O.Grain(g, (int(b[3]), int(b[2]), int(b[1])), pp[g]))
+    assert len(pp) > 128
+    for g in pp:
+        rm, rid = O.neighbour_max(g, grains, pp, (dims[2], dims[1], dims[0]), 7.0)
+        assert np.array_equal(m[g], rm.astype(np.float32)) and np.array_equal(idm[g], rid)
+        assert np.array_equal(phic[g], np.float32(0.5) * (phip[g] - m[g]))
+
+
+def test_wide_field_tiles_equal_the_others(L):
+    """A domain above the size from which physics takes 32-column tiles, made of two copies of one below it along
+    x (seed coordinates of 20 binary places, so that every displacement is the same number in both): each copy's
+    grains have the boxes and volumes of the single one's, bit for bit."""
+    nx, ny, nz, steps = 512, 320, 320, 3
+    G = nx * ny * nz // 6000
+    one = np.round(I.voronoi_seeds(9, G, (nx, ny, nz)) * 2.0 ** 20) / 2.0 ** 20
+    e = 4e-3 * I.u01(9, 7, np.arange(G))
+    res = []
+    for k in (1, 2):
+        seeds = np.concatenate([one + [nx * c, 0.0, 0.0] for c in range(k)])
+        with L.Microstructure(k * nx, ny, nz, k * G, seeds=seeds, energy=np.tile(e, k), physics=L.PHYSICS_MAGNETIC) as ms:
+            ms.step(steps, 1.0)
+            res.append((ms.grain_volumes(), ms.boxes()))
+    (v1, b1), (v2, b2) = res
+    for c in (0, 1):
+        s = slice(c * G, (c + 1) * G)
+        assert np.array_equal(v2[s], v1)
+        assert np.array_equal(b2[s][:, [0, 2, 3, 4, 5, 6]], b1[:, [0, 2, 3, 4, 5, 6]])
+        assert np.array_equal((b2[s][:, 1] - nx * c) % (2 * nx) % nx, b1[:, 1] % nx)
