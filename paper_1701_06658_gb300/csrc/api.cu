@@ -587,6 +587,7 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     c->B.prev = c->d_boxes;
     c->B.cur = c->d_boxes + G;
     c->B.use_passes = cfg_in->exec == LSGG_EXEC_BATCHED ? 1 : 0;
+    c->B.phys_kind = cfg_in->physics;
     c->B.bf16 = cfg_in->storage == LSGG_STORAGE_BF16 ? 1 : 0;
     c->B.redist = cfg_in->redist;
     c->B.wait_limit = kWaitIters;

@@ -168,6 +168,7 @@ __device__ __forceinline__ float key_val(unsigned long long k, float eps) {
 struct StepBuffers {
     Domain dom;
     int n_boxes;
+    int phys_kind;                  // LSGG_PHYSICS_* (the launch shapes of the z pass)
     int bf16;                       // X holds BF16 (LSGG_STORAGE_BF16); arithmetic stays FP32
     int redist;                     // LSGG_REDIST_*: TAXICAB by the pass kernels; GODUNOV and HARTMANN
                                     // by Jacobi sweeps over the boxes' columns

@@ -390,11 +390,11 @@ constexpr int kZHash = 2 * kPoolKeys;
 static_assert((kZHash & (kZHash - 1)) == 0, "pair hash slots: a power of two");
 __device__ __forceinline__ unsigned zhash(int j) { return ((unsigned)j * 2654435761u) >> 22; }
 static_assert((1u << 10) == kZHash, "zhash yields the slot bits of kZHash");
-__device__ __forceinline__ int zslot(const int* hk, int j) {
+__device__ __forceinline__ int zslot(const int2* hash, int j) {
     unsigned h = zhash(j);
 #pragma unroll 1
     for (int p = 0; p < kZHash; ++p) {
-        const int k = hk[h];
+        const int k = hash[h].x;
         if (k == j) return (int)h;
         if (k < 0) return -1;
         h = (h + 1) & (kZHash - 1);
@@ -402,93 +402,209 @@ __device__ __forceinline__ int zslot(const int* hk, int j) {
     return -1;
 }
 
-constexpr int kColumnRadius = 5;   // the physics z pass keeps its column in registers at this radius
+constexpr int kColumnRadius = 5;   // radius for which the physics z pass has its own column code
 
 // Read-Shockley weights of a pair missing from the box's hash (a list that
-// did not fit the pool): out of line, so that the unrolled column below
-// keeps one call per cell instead of the FP64 evaluation.
+// did not fit the pool): out of line, so that the unrolled loop below keeps
+// one call per cell instead of the FP64 evaluation.
 __device__ __noinline__ void rs_pair_out_of_line(const PhysicsDev& phys, int i, int j, float& w, float& m) {
     rs_pair(phys, i, j, w, m);
 }
 
-// z pass with the velocity correction of Eq. (10) for one column of nz <= NZ
-// cells on a non-periodic axis: the z convolution from the column in
-// registers (as conv_column), then per group of eight cells the previous
-// step's phi and pair ids (old layout; -eps and no pair outside the old box)
-// loaded together, the bulk energies e_j loaded together, and the blend
-// phi + w (c - phi) + M (e_j - e_i) dt with w and M from the box's pair hash
-// (Read-Shockley) or 1 (magnetic); cells without a pair take c.
-template <int R, int NZ>
-__device__ __forceinline__ void conv_column_phys(const StepBuffers& B, const PhysicsDev& phys, const float* zc, float* yc,
-                                                 int nz, int ps, const float (&g)[2 * R + 1], float cconst, float eps,
-                                                 long long o_old, int ps_old, int ozl0, int onz, int dnz, bool in_old,
-                                                 int b, float ei, bool rs, const int* hk, const float* hw,
-                                                 const float* hm) {
-    constexpr int W = 2 * R + 1;
-    constexpr int G8 = 8;
-    float r[NZ + 2 * R];
+// z pass with the velocity correction of Eq. (10) for one column on a
+// non-periodic axis, any length.  The convolution runs in transposed form: a
+// plane's value enters the partial sums of the 2 R outputs that still need it
+// (a[i] = fma(g, v, a[i + 1]), which moves the sums along without copies) and
+// completes one; an output takes its taps in the order k = 0 .. 2 R from 0, as
+// conv_column does.  Ten sums instead of the whole column leave the registers
+// to a batch of kZB planes' loads -- the plane, the previous step's phi and
+// pair id (old layout; -eps and no pair outside the old box), then the bulk
+// energies -- all in flight together, at four CTAs per SM instead of two.
+// Cells without a pair take the convolution c, others phi + w (c - phi) + M
+// (e_j - e_i) dt: Read-Shockley (RS) with w from the box's pair hash and no
+// bulk term, magnetic with w = M = 1.
+template <int R, bool RS>
+__device__ __forceinline__ void conv_fir_phys(const StepBuffers& B, const PhysicsDev& phys, const float* zc, float* yc,
+                                              int nz, int ps, const float (&g)[2 * R + 1], float cconst, float eps,
+                                              long long o_old, int ps_old, int ozl0, int onz, int dnz, bool in_old, float ei,
+                                              const int2* hash) {
+    float a[2 * R];
+    // planes -R .. -1 are cconst: the outputs z = 0 .. R - 1 start with R - z of its taps
+    {
+        float c = 0.0f;
 #pragma unroll
-    for (int k = 0; k < R; ++k) r[k] = cconst;
+        for (int k = 0; k < R; ++k) {
+            c = fmaf(g[k], cconst, c);
+            a[2 * R - 1 - k] = c;
+            a[k] = 0.0f;                                   // outputs before the box
+        }
+    }
+    const bool bf16 = B.bf16 != 0;
+    const float* const xo = B.X + (bf16 ? 0 : o_old);
+    const __nv_bfloat16* const xb = reinterpret_cast<const __nv_bfloat16*>(B.X) + o_old;
+    const int* const jo = B.IDF + o_old;
+    for (int base = 0; base < nz + R; base += kZB) {
+        float v[kZB], p0[kZB], ej[RS ? 1 : kZB];
+        int jj[kZB];
 #pragma unroll
-    for (int z = 0; z < NZ; ++z) r[R + z] = __ldg(zc + (long long)min(z, nz - 1) * ps);
+        for (int u = 0; u < kZB; ++u)
+            v[u] = base + u < nz ? __ldg(zc + (size_t)((unsigned)(base + u) * (unsigned)ps)) : cconst;
 #pragma unroll
-    for (int z = 0; z < NZ + R; ++z)
-        if (z >= nz) r[R + z] = cconst;
-#pragma unroll
-    for (int z0 = 0; z0 < NZ; z0 += G8) {
-        if (z0 >= nz) break;                               // uniform: one box per CTA item
-        float p0[G8], ej[G8];
-        int jj[G8];
-#pragma unroll
-        for (int u = 0; u < G8; ++u) {
-            const int z = z0 + u;
-            int ozl = ozl0 + z;                            // ozl0 + z < 2 N_z
+        for (int u = 0; u < kZB; ++u) {
+            const int zo = base + u - R;
+            int ozl = ozl0 + zo;                           // ozl0 + zo < 2 N_z
             if (ozl >= dnz) ozl -= dnz;
-            const bool ok = z < nz && in_old && ozl < onz;
-            const long long o = o_old + (long long)(ok ? ozl : 0) * ps_old;
-            p0[u] = ok ? ld_state(B, o) : -eps;
-            jj[u] = ok ? B.IDF[o] : -1;
+            const bool ok = zo >= 0 && zo < nz && in_old && ozl < onz;
+            const unsigned o = ok ? (unsigned)ozl * (unsigned)ps_old : 0u;
+            jj[u] = ok ? jo[o] : -1;
+            p0[u] = !ok ? -eps : (bf16 ? __bfloat162float(xb[o]) : xo[o]);
+        }
+        if constexpr (!RS) {
+#pragma unroll
+            for (int u = 0; u < kZB; ++u) ej[u] = jj[u] >= 0 ? __ldg(phys.energy + jj[u]) : 0.0f;
         }
 #pragma unroll
-        for (int u = 0; u < G8; ++u) ej[u] = phys.energy && jj[u] >= 0 ? __ldg(phys.energy + jj[u]) : 0.0f;
+        for (int u = 0; u < kZB; ++u) {
+            float val = fmaf(g[2 * R], v[u], a[0]);
 #pragma unroll
-        for (int u = 0; u < G8; ++u) {
-            const int z = z0 + u;
-            if (z >= nz) break;
-            float acc = 0.0f;
-#pragma unroll
-            for (int k = 0; k < W; ++k) acc = fmaf(g[k], r[z + k], acc);
-            float val = acc;
+            for (int i = 0; i < 2 * R - 1; ++i) a[i] = fmaf(g[2 * R - 1 - i], v[u], a[i + 1]);
+            a[2 * R - 1] = fmaf(g[0], v[u], 0.0f);
+            const int zo = base + u - R;
+            if (zo < 0 || zo >= nz) continue;
             const int j = jj[u];
             if (j >= 0) {
-                float w = 1.0f, m = 1.0f;
-                if (rs) {
-                    const int h = zslot(hk, j);
-                    if (h >= 0) {
-                        w = hw[h];
-                        m = hm[h];
-                    } else {
-                        rs_pair_out_of_line(phys, b, j, w, m);
+                if constexpr (RS) {
+                    // the list holds every id of the box's ID-field; at most
+                    // half full, so an empty slot would end the search
+                    unsigned h = zhash(j);
+                    int2 e = hash[h];
+                    while (e.x != j && e.x >= 0) {
+                        h = (h + 1) & (kZHash - 1);
+                        e = hash[h];
                     }
+                    val = fmaf(__int_as_float(e.y), val - p0[u], p0[u]);
+                } else {
+                    val = fmaf(ej[u] - ei, phys.dt, p0[u] + (val - p0[u]));
                 }
-                float bulk = 0.0f;
-                if (phys.energy) bulk = m * (ej[u] - ei) * phys.dt;
-                val = p0[u] + w * (acc - p0[u]) + bulk;
             }
-            yc[(long long)z * ps] = fminf(fmaxf(val, -eps), eps);
+            yc[(size_t)((unsigned)zo * (unsigned)ps)] = fminf(fmaxf(val, -eps), eps);
         }
     }
 }
 
-template <int R, bool PHYS, bool GRP>
-__global__ void __launch_bounds__(kColThreads, PHYS ? 2 : (R < 5 ? 4 : 3))
-p_conv_z(StepBuffers B1, GroupRef grp, Taps taps, PhysicsDev phys, int tier) {
+// The z pass of one column in its general form (periodic or long columns; with
+// PHYS, pairs from the anisotropy map, from the fixed table of a box whose list
+// did not fit the pool, or at another radius): a window over the column, its
+// planes loaded in batches.  Out of line: the Read-Shockley evaluation would
+// otherwise cost the common form its registers.
+template <int R, bool PHYS>
+__device__ __noinline__ void conv_z_general(const StepBuffers& B, const PhysicsDev& phys, const Taps& taps,
+                                            const PairTable& tab, const int2* hash, int hash_n, int b, int c) {
+    constexpr int W = 2 * R + 1;
+    float g[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) g[k] = taps.g[k];
+    const Domain D = B.dom;
+    const float cconst = conv_xy_of_const<R>(g, -D.eps);
+    const bool rs = PHYS && phys.kind == LSGG_PHYSICS_READ_SHOCKLEY;
+    const Box nb = B.cur[b], ob = B.prev[b];
+    const int nx = nb.nx, ny = nb.ny, nz = nb.nz;
+    const bool fz = nz == D.nz;
+    const int ps = plane_stride(nx, ny), ps_old = plane_stride(ob.nx, ob.ny);
+    const float* zc = B.Z + nb.off + c;
+    float* yc = B.Y + nb.off + c;
+    int oxl = 0, oyl = 0;
+    bool in_old_xy = false;
+    if (PHYS) {
+        const int y = c / nx, x = c - y * nx;
+        oxl = wrap_near(nb.ox + x - ob.ox, D.nx);
+        oyl = wrap_near(nb.oy + y - ob.oy, D.ny);
+        in_old_xy = oxl < ob.nx && oyl < ob.ny;
+    }
+    PairCache pcache;
+    const float ei = PHYS && phys.energy ? phys.energy[b] : 0.0f;
+    float win[W];                                      // planes zo-R .. zo+R
+#pragma unroll
+    for (int k = 0; k < W; ++k) win[k] = cconst;
+    const int n_in = nz + 2 * R;                       // input planes -R .. nz+R-1
+    for (int base = 0; base < n_in; base += kZB) {
+        float v[kZB];
+#pragma unroll
+        for (int u = 0; u < kZB; ++u) {
+            const int zin = base + u - R;
+            v[u] = cconst;
+            if (base + u < n_in) {
+                if (fz) v[u] = zc[(long long)pmod(zin, nz) * ps];
+                else if (zin >= 0 && zin < nz) v[u] = zc[(long long)zin * ps];
+            }
+        }
+        // the previous step's phi and ID-field of this batch's output planes
+        float phi0[PHYS ? kZB : 1];
+        int jn[PHYS ? kZB : 1];
+        if (PHYS) {
+#pragma unroll
+            for (int u = 0; u < kZB; ++u) {
+                const int zo = base + u - 2 * R;
+                const int ozl = wrap_near(nb.oz + zo - ob.oz, D.nz);
+                phi0[u] = -D.eps;
+                jn[u] = -1;
+                if (zo >= 0 && zo < nz && in_old_xy && ozl < ob.nz) {
+                    const long long o = ob.off + (long long)ozl * ps_old + (long long)oyl * ob.nx + oxl;
+                    phi0[u] = ld_state(B, o);
+                    jn[u] = B.IDF[o];
+                }
+                if (phys.pair_map && zo >= 0 && zo < nz) jn[u] = phys.pair_map[nb.off + (long long)zo * ps + c];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kZB; ++u) {
+            if (base + u >= n_in) break;
+#pragma unroll
+            for (int k = 0; k < W - 1; ++k) win[k] = win[k + 1];
+            win[W - 1] = v[u];
+            const int zo = base + u - 2 * R;
+            if (zo < 0) continue;
+            float acc = 0.0f;
+#pragma unroll
+            for (int k = 0; k < W; ++k) acc = fmaf(g[k], win[k], acc);
+            float val = acc;
+            if (PHYS && hash_n >= 0) {
+                // Eq. (10) with the pair's w from the box's hash (Read-Shockley:
+                // no bulk term; the arithmetic of pair_blend)
+                const int j = jn[u];
+                if (j >= 0) {
+                    const int h = zslot(hash, j);
+                    float w = 1.0f;
+                    if (h >= 0) {
+                        w = __int_as_float(hash[h].y);
+                    } else {                               // not in the box's list: direct
+                        float m;
+                        rs_pair_out_of_line(phys, b, j, w, m);
+                    }
+                    val = fmaf(w, acc - phi0[u], phi0[u]);
+                }
+            } else if (PHYS) {
+                val = pair_blend_cached(phys, tab, b, jn[u], phi0[u], acc, ei, pcache);
+            }
+            val = fminf(fmaxf(val, -D.eps), D.eps);
+            yc[(long long)zo * ps] = val;
+        }
+    }
+}
+
+// KIND: LSGG_PHYSICS_*.  CTAs per SM: Read-Shockley four (512^3: 3.56 ms, 3.75
+// at three), magnetic three, whose gathered energies spill at four (384^3:
+// 1.48 ms, 2.50 at four); GB300.
+template <int R, int KIND, bool GRP>
+__global__ void __launch_bounds__(kColThreads, KIND == LSGG_PHYSICS_READ_SHOCKLEY || R < 5 ? 4 : 3)
+p_conv_z(const __grid_constant__ StepBuffers B1, GroupRef grp, const __grid_constant__ Taps taps,
+         const __grid_constant__ PhysicsDev phys, int tier) {
+    constexpr bool PHYS = KIND != LSGG_PHYSICS_IDEAL;
     static_assert(!(GRP && PHYS), "step groups run ideal growth");
     constexpr int W = 2 * R + 1;
     __shared__ int s_tj[PHYS ? kNbCap : 1];
     __shared__ float s_tw[PHYS ? kNbCap : 1], s_tm[PHYS ? kNbCap : 1];
-    __shared__ int s_hk[PHYS ? kZHash : 1];
-    __shared__ float s_hw[PHYS ? kZHash : 1], s_hm[PHYS ? kZHash : 1];
+    __shared__ int2 s_h[PHYS ? kZHash : 1];                // the pair hash: id (-1: empty), w
     __shared__ int s_gb[GRP ? kMaxGroup + 1 : 1];
     if (!GRP && halted(B1)) return;
     float g[W];
@@ -497,7 +613,7 @@ p_conv_z(StepBuffers B1, GroupRef grp, Taps taps, PhysicsDev phys, int tier) {
     const float cconst1 = GRP ? 0.0f : conv_xy_of_const<R>(g, -B1.dom.eps);
     const int n_items = GRP ? group_scan(grp, kItemChunks, tier, true, s_gb) : B1.st->n_chunks[tier];
     const int2* items = GRP ? nullptr : B1.chunk_items + B1.st->chunk_base[tier];
-    const bool rs = PHYS && phys.kind == LSGG_PHYSICS_READ_SHOCKLEY;
+    constexpr bool rs = KIND == LSGG_PHYSICS_READ_SHOCKLEY;
     const bool pooled = PHYS && phys.pool_ent[0] != nullptr && phys.pair_map == nullptr;
     // this step's pool (the parity of the steps done)
     const bool odd = pooled && (B1.st->steps_done & 1);
@@ -509,8 +625,6 @@ p_conv_z(StepBuffers B1, GroupRef grp, Taps taps, PhysicsDev phys, int tier) {
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         int local;
         const StepBuffers& B = member<GRP>(B1, grp, s_gb, item, local);
-        const Domain D = B.dom;
-        const float cconst = GRP ? conv_xy_of_const<R>(g, -D.eps) : cconst1;
         const int2 it = list_item<GRP>(B, items, kItemChunks, tier, item, local);
         const int b = it.x;
         if (PHYS && (rs || pooled) && b != last_b) {       // uniform across the CTA
@@ -522,15 +636,14 @@ p_conv_z(StepBuffers B1, GroupRef grp, Taps taps, PhysicsDev phys, int tier) {
                 if (pb.y >= 0 && pb.y <= kZHash / 2) hash_n = pb.y;
             }
             if (hash_n >= 0) {
-                for (int k = threadIdx.x; k < kZHash; k += blockDim.x) s_hk[k] = -1;
+                for (int k = threadIdx.x; k < kZHash; k += blockDim.x) s_h[k].x = -1;
                 __syncthreads();
                 const int2 pb = pool_box[b];
                 for (int k = threadIdx.x; k < hash_n; k += blockDim.x) {
                     const int4 e = pool_ent[pb.x + k];
                     unsigned h = zhash(e.x);
-                    while (atomicCAS(&s_hk[h], -1, e.x) != -1) h = (h + 1) & (kZHash - 1);
-                    s_hw[h] = __int_as_float(e.y);
-                    s_hm[h] = __int_as_float(e.z);
+                    while (atomicCAS(&s_h[h].x, -1, e.x) != -1) h = (h + 1) & (kZHash - 1);
+                    s_h[h].y = e.y;
                 }
             } else if (rs) {
                 tab = load_pair_table(phys, b, s_tj, s_tw, s_tm);
@@ -538,124 +651,43 @@ p_conv_z(StepBuffers B1, GroupRef grp, Taps taps, PhysicsDev phys, int tier) {
             __syncthreads();
         }
         last_b = b;
-        const Box nb = B.cur[b], ob = B.prev[b];
+        const Box nb = B.cur[b];
         const int nx = nb.nx, ny = nb.ny, nz = nb.nz;
-        const bool fz = nz == D.nz;
+        const int dnx = B.dom.nx, dny = B.dom.ny, dnz = B.dom.nz;
+        const float eps = B.dom.eps;
+        const bool fz = nz == dnz;
         const int c = it.y * kPassChunk + threadIdx.x;
         if (c >= nx * ny) continue;
         const int ps = plane_stride(nx, ny);
         const float* zc = B.Z + nb.off + c;
         float* yc = B.Y + nb.off + c;
-        int oxl = 0, oyl = 0;
-        bool in_old_xy = false;
-        if (PHYS) {
-            const int y = c / nx, x = c - y * nx;
-            oxl = wrap_near(nb.ox + x - ob.ox, D.nx);
-            oyl = wrap_near(nb.oy + y - ob.oy, D.ny);
-            in_old_xy = oxl < ob.nx && oyl < ob.ny;
-        }
-        if (!PHYS && !fz && nz <= 64) {                    // uniform across the CTA (one box per item)
-            if (nz <= 16) conv_column<R, 16>(zc, yc, nz, ps, g, cconst, D.eps);
-            else if (nz <= 32) conv_column<R, 32>(zc, yc, nz, ps, g, cconst, D.eps);
-            else if (nz <= 48) conv_column<R, 48>(zc, yc, nz, ps, g, cconst, D.eps);
-            else conv_column<R, 64>(zc, yc, nz, ps, g, cconst, D.eps);
-            continue;
-        }
-        const int ps_old = plane_stride(ob.nx, ob.ny);
-        // the paper's radius (the column code is instantiated for it alone)
-        if constexpr (PHYS && R == kColumnRadius) {
-            if (!fz && nz <= 64 && !phys.pair_map && (!rs || hash_n >= 0)) {
-                // uniform across the CTA
-                const long long o_old = ob.off + (long long)oyl * ob.nx + oxl;
-                const int ozl0 = wrap_near(nb.oz - ob.oz, D.nz);
-                const float ei = phys.energy ? phys.energy[b] : 0.0f;
-                if (nz <= 16)
-                    conv_column_phys<R, 16>(B, phys, zc, yc, nz, ps, g, cconst, D.eps, o_old, ps_old, ozl0, ob.nz, D.nz,
-                                            in_old_xy, b, ei, rs, s_hk, s_hw, s_hm);
-                else if (nz <= 32)
-                    conv_column_phys<R, 32>(B, phys, zc, yc, nz, ps, g, cconst, D.eps, o_old, ps_old, ozl0, ob.nz, D.nz,
-                                            in_old_xy, b, ei, rs, s_hk, s_hw, s_hm);
-                else if (nz <= 48)
-                    conv_column_phys<R, 48>(B, phys, zc, yc, nz, ps, g, cconst, D.eps, o_old, ps_old, ozl0, ob.nz, D.nz,
-                                            in_old_xy, b, ei, rs, s_hk, s_hw, s_hm);
-                else
-                    conv_column_phys<R, 64>(B, phys, zc, yc, nz, ps, g, cconst, D.eps, o_old, ps_old, ozl0, ob.nz, D.nz,
-                                            in_old_xy, b, ei, rs, s_hk, s_hw, s_hm);
+        // every branch is uniform across the CTA (one box per item)
+        if constexpr (!PHYS) {
+            if (!fz && nz <= 64) {
+                const float cconst = GRP ? conv_xy_of_const<R>(g, -eps) : cconst1;
+                if (nz <= 16) conv_column<R, 16>(zc, yc, nz, ps, g, cconst, eps);
+                else if (nz <= 32) conv_column<R, 32>(zc, yc, nz, ps, g, cconst, eps);
+                else if (nz <= 48) conv_column<R, 48>(zc, yc, nz, ps, g, cconst, eps);
+                else conv_column<R, 64>(zc, yc, nz, ps, g, cconst, eps);
                 continue;
             }
         }
-        PairCache pcache;
-        const float ei = PHYS && phys.energy ? phys.energy[b] : 0.0f;
-        float win[W];                                      // planes zo-R .. zo+R
-#pragma unroll
-        for (int k = 0; k < W; ++k) win[k] = cconst;
-        const int n_in = nz + 2 * R;                       // input planes -R .. nz+R-1
-        for (int base = 0; base < n_in; base += kZB) {
-            float v[kZB];
-#pragma unroll
-            for (int u = 0; u < kZB; ++u) {
-                const int zin = base + u - R;
-                v[u] = cconst;
-                if (base + u < n_in) {
-                    if (fz) v[u] = zc[(long long)pmod(zin, nz) * ps];
-                    else if (zin >= 0 && zin < nz) v[u] = zc[(long long)zin * ps];
-                }
-            }
-            // the previous step's phi and ID-field of this batch's output planes
-            float phi0[PHYS ? kZB : 1];
-            int jn[PHYS ? kZB : 1];
-            if (PHYS) {
-#pragma unroll
-                for (int u = 0; u < kZB; ++u) {
-                    const int zo = base + u - 2 * R;
-                    const int ozl = wrap_near(nb.oz + zo - ob.oz, D.nz);
-                    phi0[u] = -D.eps;
-                    jn[u] = -1;
-                    if (zo >= 0 && zo < nz && in_old_xy && ozl < ob.nz) {
-                        const long long o = ob.off + (long long)ozl * ps_old + (long long)oyl * ob.nx + oxl;
-                        phi0[u] = ld_state(B, o);
-                        jn[u] = B.IDF[o];
-                    }
-                    if (phys.pair_map && zo >= 0 && zo < nz) jn[u] = phys.pair_map[nb.off + (long long)zo * ps + c];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kZB; ++u) {
-                if (base + u >= n_in) break;
-#pragma unroll
-                for (int k = 0; k < W - 1; ++k) win[k] = win[k + 1];
-                win[W - 1] = v[u];
-                const int zo = base + u - 2 * R;
-                if (zo < 0) continue;
-                float acc = 0.0f;
-#pragma unroll
-                for (int k = 0; k < W; ++k) acc = fmaf(g[k], win[k], acc);
-                float val = acc;
-                if (PHYS && hash_n >= 0) {
-                    // Eq. (10) with the pair's w and M from the box's hash
-                    // (the arithmetic of pair_blend)
-                    const int j = jn[u];
-                    if (j >= 0) {
-                        const int h = zslot(s_hk, j);
-                        float w = 1.0f, m = 1.0f;
-                        if (h >= 0) {
-                            w = s_hw[h];
-                            m = s_hm[h];
-                        } else if (rs) {                       // not in the box's list: direct
-                            rs_pair_out_of_line(phys, b, j, w, m);
-                        }
-                        const float ej = phys.energy ? phys.energy[j] : 0.0f;
-                        float bulk = 0.0f;
-                        if (phys.energy) bulk = m * (ej - ei) * phys.dt;
-                        val = phi0[u] + w * (acc - phi0[u]) + bulk;
-                    }
-                } else if (PHYS) {
-                    val = pair_blend_cached(phys, tab, b, jn[u], phi0[u], acc, ei, pcache);
-                }
-                val = fminf(fmaxf(val, -D.eps), D.eps);
-                yc[(long long)zo * ps] = val;
+        // the paper's radius (the column code is instantiated for it alone)
+        if constexpr (PHYS && R == kColumnRadius) {
+            if (!fz && !phys.pair_map && (rs ? hash_n >= 0 : phys.energy != nullptr)) {
+                const Box ob = B.prev[b];
+                const int ps_old = plane_stride(ob.nx, ob.ny);
+                const int y = c / nx, x = c - y * nx;
+                const int oxl = wrap_near(nb.ox + x - ob.ox, dnx), oyl = wrap_near(nb.oy + y - ob.oy, dny);
+                const bool in_old = oxl < ob.nx && oyl < ob.ny;
+                const long long o_old = ob.off + (in_old ? (long long)oyl * ob.nx + oxl : 0);
+                const int ozl0 = wrap_near(nb.oz - ob.oz, dnz);
+                conv_fir_phys<R, rs>(B, phys, zc, yc, nz, ps, g, cconst1, eps, o_old, ps_old, ozl0, ob.nz, dnz, in_old,
+                                     rs ? 0.0f : phys.energy[b], s_h);
+                continue;
             }
         }
+        conv_z_general<R, PHYS>(B, phys, taps, tab, s_h, hash_n, b, c);
     }
 }
 
@@ -2156,7 +2188,7 @@ struct PassFns {
 };
 
 template <int R, bool GRP = false>
-static PassFns pass_fns_r(bool phys) {
+static PassFns pass_fns_r(int kind) {
     static_assert(kTiers == 5, "one instantiation per tier side");
     PassFns f;
     f.conv_xy[0] = reinterpret_cast<const void*>(p_conv_xy<R, 32, kConvThreads[0], GRP>);
@@ -2164,9 +2196,10 @@ static PassFns pass_fns_r(bool phys) {
     f.conv_xy[2] = reinterpret_cast<const void*>(p_conv_xy<R, 48, kConvThreads[2], GRP>);
     f.conv_xy[3] = reinterpret_cast<const void*>(p_conv_xy<R, 64, kConvThreads[3], GRP>);
     f.conv_xy[4] = reinterpret_cast<const void*>(p_conv_xy_big<R, GRP>);
-    if constexpr (GRP) f.conv_z = reinterpret_cast<const void*>(p_conv_z<R, false, true>);
-    else f.conv_z = phys ? reinterpret_cast<const void*>(p_conv_z<R, true, false>)
-                         : reinterpret_cast<const void*>(p_conv_z<R, false, false>);
+    if constexpr (GRP) f.conv_z = reinterpret_cast<const void*>(p_conv_z<R, LSGG_PHYSICS_IDEAL, true>);
+    else f.conv_z = kind == LSGG_PHYSICS_READ_SHOCKLEY ? reinterpret_cast<const void*>(p_conv_z<R, LSGG_PHYSICS_READ_SHOCKLEY, false>)
+                    : kind == LSGG_PHYSICS_MAGNETIC    ? reinterpret_cast<const void*>(p_conv_z<R, LSGG_PHYSICS_MAGNETIC, false>)
+                                                       : reinterpret_cast<const void*>(p_conv_z<R, LSGG_PHYSICS_IDEAL, false>);
     f.redist_xy[0] = reinterpret_cast<const void*>(p_redist_xy<32, kRedistThreads[0], GRP>);
     f.redist_xy[1] = reinterpret_cast<const void*>(p_redist_xy<40, kRedistThreads[1], GRP>);
     f.redist_xy[2] = reinterpret_cast<const void*>(p_redist_xy<48, kRedistThreads[2], GRP>);
@@ -2175,22 +2208,23 @@ static PassFns pass_fns_r(bool phys) {
     return f;
 }
 
-static bool pass_fns(int R, bool phys, PassFns* f) {
+static bool pass_fns(int R, int kind, PassFns* f) {
     switch (R) {
-        case 1: *f = pass_fns_r<1>(phys); return true;
-        case 2: *f = pass_fns_r<2>(phys); return true;
-        case 3: *f = pass_fns_r<3>(phys); return true;
-        case 4: *f = pass_fns_r<4>(phys); return true;
-        case 5: *f = pass_fns_r<5>(phys); return true;
-        case 6: *f = pass_fns_r<6>(phys); return true;
-        case 7: *f = pass_fns_r<7>(phys); return true;
+        case 1: *f = pass_fns_r<1>(kind); return true;
+        case 2: *f = pass_fns_r<2>(kind); return true;
+        case 3: *f = pass_fns_r<3>(kind); return true;
+        case 4: *f = pass_fns_r<4>(kind); return true;
+        case 5: *f = pass_fns_r<5>(kind); return true;
+        case 6: *f = pass_fns_r<6>(kind); return true;
+        case 7: *f = pass_fns_r<7>(kind); return true;
         default: return false;
     }
 }
 
 cudaError_t configure_passes(StepBuffers& B) {
     PassFns fn, fn_ideal;
-    if (!pass_fns(B.dom.radius, true, &fn) || !pass_fns(B.dom.radius, false, &fn_ideal)) return cudaErrorInvalidValue;
+    if (!pass_fns(B.dom.radius, B.phys_kind, &fn) || !pass_fns(B.dom.radius, LSGG_PHYSICS_IDEAL, &fn_ideal))
+        return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     for (int t = 0; t < kTiers; ++t) {
         B.tier_side[t] = kTierSide[t];
@@ -2239,7 +2273,7 @@ cudaError_t configure_passes(StepBuffers& B) {
 cudaError_t launch_passes(const StepBuffers& B, int which, int tier, const Taps& taps, const PhysicsDev& phys,
                           const DebugOut& dbg, cudaStream_t s, cudaEvent_t* pass_ev) {
     PassFns fn;
-    if (!pass_fns(taps.radius, phys.kind != LSGG_PHYSICS_IDEAL, &fn)) return cudaErrorInvalidValue;
+    if (!pass_fns(taps.radius, phys.kind, &fn)) return cudaErrorInvalidValue;
     const int* g = B.pgrid[tier];
     StepBuffers bb = B;
     Taps tp = taps;
@@ -2303,7 +2337,7 @@ static GroupShapes g_group_shapes{};
 cudaError_t launch_passes_group(const StepBuffers& B0, const GroupRef& grp, int which, int tier, const Taps& taps,
                                 cudaStream_t s) {
     if (taps.radius != kGroupRadius) return cudaErrorInvalidValue;
-    const PassFns fn = pass_fns_r<kGroupRadius, true>(false);
+    const PassFns fn = pass_fns_r<kGroupRadius, true>(LSGG_PHYSICS_IDEAL);
     const int* g = g_group_shapes.pgrid[tier];
     StepBuffers bb = B0;
     GroupRef gr = grp;
@@ -2332,7 +2366,7 @@ cudaError_t launch_passes_group(const StepBuffers& B0, const GroupRef& grp, int 
 }
 
 cudaError_t configure_group_kernels(int n_sm) {
-    const PassFns fn = pass_fns_r<kGroupRadius, true>(false);
+    const PassFns fn = pass_fns_r<kGroupRadius, true>(LSGG_PHYSICS_IDEAL);
     GroupShapes sh{};
     sh.n_sm = n_sm;
     for (int t = 0; t < kTiers; ++t) {

@@ -137,3 +137,35 @@ def test_wide_field_tiles_equal_the_others(L):
         assert np.array_equal(v2[s], v1)
         assert np.array_equal(b2[s][:, [0, 2, 3, 4, 5, 6]], b1[:, [0, 2, 3, 4, 5, 6]])
         assert np.array_equal((b2[s][:, 1] - nx * c) % (2 * nx) % nx, b1[:, 1] % nx)
+
+
+@pytest.mark.parametrize("kind", ["read_shockley", "magnetic"])
+@pytest.mark.parametrize("dims,G,bf16", [
+    ((36, 36, 160), 6, False),       # columns of up to a hundred cells beside short ones
+    ((44, 40, 52), 40, False),       # column lengths on both sides of a batch of eight
+    ((44, 40, 52), 40, True),        # previous phi in BF16
+    ((24, 24, 24), 6, False),        # periodic columns: the general form
+])
+def test_physics_z_pass_against_the_oracle(L, kind, dims, G, bf16):
+    """phi_p of the second step (previous boxes and ID-field of the first) within the FP32 tolerance of the
+    parity tests, 3e-5."""
+    from oracle import lsgg_oracle as O
+    from tests.parity import oracle_from_gpu
+    quats, e = I.random_quaternions(12, G), 4e-2 * I.u01(12, 7, np.arange(G))
+    kw = {"quats": quats, "physics": L.PHYSICS_READ_SHOCKLEY} if kind == "read_shockley" else \
+        {"energy": e, "physics": L.PHYSICS_MAGNETIC}
+    ph = O.read_shockley_physics(quats) if kind == "read_shockley" else O.isotropic_physics(e)
+    shape = (dims[2], dims[1], dims[0])
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(12, G, dims), storage=L.STORAGE_BF16 if bf16 else
+                          L.STORAGE_FP32, **kw) as ms:
+        old, (_, _, idm, _, _) = ms.debug_step(1.0)
+        boxes, phi = ms.boxes(), ms.phi()
+        ref = oracle_from_gpu(shape, boxes, phi, None, ph)
+        for g in phi:                                # the first step's ID-field on the boxes after it
+            was = O.Grain(g, (int(old[g, 3]), int(old[g, 2]), int(old[g, 1])), idm[g].astype(np.float64))
+            ref.grains[g].idf = O.sample(was, O.box_positions(ref.grains[g], shape), shape, -1)[0].astype(np.int64)
+        _, (phip, *_rest) = ms.debug_step(1.0)
+    taps = O.heat_kernel_taps(1.0, 5)
+    for g in phip:
+        want = O.predict(ref.grains[g], shape, taps, 7.0, ph, 1.0)
+        assert np.max(np.abs(phip[g] - want)) <= 3e-5, g
