@@ -80,52 +80,68 @@ __device__ __forceinline__ float conv_xy_of_const(const float (&g)[2 * R + 1], f
 }
 
 // ---------------------------------------------------------------------------
-// pass 1: xy convolution of one plane
+// pass 1: xy convolution, two planes at a time
 // ---------------------------------------------------------------------------
-// A CTA of NT threads takes one (box, plane) item at a time:
-//   fetch   the plane of phi in the box's previous layout (contiguous,
-//           16-byte aligned) arrives in a raw slot by a bulk copy, issued
-//           while the CTA still works on the item before;
-//   stage   raw -> padded grid P in the new layout (-eps outside the old
-//           box), a thread per group of four cells of a padded row; rows
-//           outside the old box are left unstaged;
+// A CTA of NT threads takes one (box, slab) item at a time and its planes in
+// pairs (z, z + 1), a cell of both planes as one 64-bit pair: staging, window
+// loads, index arithmetic and the packed FMAs (fma.rn.f32x2, two rounded FMAs
+// in one instruction) serve both.
+//   fetch   the two planes of phi in the box's previous layout (contiguous,
+//           16-byte aligned) arrive in raw slots by bulk copies, issued while
+//           the CTA still works on the pair before;
+//   stage   raw -> grid P of pairs, the old box's rows with their columns in
+//           the new layout, padded (-eps outside the old box); a warp per row,
+//           a lane per two cells;
 //   x pass  each thread convolves 4 consecutive cells of one padded row from
 //           16-byte shared loads -> grid XC (all padded rows; a row outside
-//           the old box is the FMA chain over -eps, written directly);
+//           the old box is the FMA chain over -eps, written directly); lanes
+//           along the rows, whose pitch is an odd number of 16-byte words, so
+//           that neither loads nor stores conflict;
 //   y pass  each thread convolves 4 consecutive rows of one column from
 //           shared loads of XC and stores them (lanes along x: coalesced).
 // The FMA order of both passes is the one conv_xy_of_const repeats.  Every
 // wait on a copy is bounded (LSGG_ERR_TIMEOUT, halt, drain, return).
 //
+// Measured on GB300: 256^3 / 5000 grains 0.607 ms plane by plane with scalar
+// FMAs (92 thread instructions a cell, 71 % of the issue slots), 0.479 ms in
+// pairs (about 45 a cell); 512^3 Read-Shockley 3.86 and 3.20 ms.  What bounds
+// it now is the latency of shared-memory loads and FMA chains at about 20
+// warps per SM: the grids' shared memory allows no more, and more threads a
+// CTA leave the last round of its tasks emptier (256^3: 0.485 ms at 192
+// threads, side 40).
+//
 // The sizes below are the one definition of the layout: the kernel's
 // offsets and the launch's dynamic shared-memory size both derive from them.
-// padded rows; 16-byte loads per x window of 4 outputs; pitch of P (room for
-// the last group's window); pitch of XC; rows of XC (3 spare rows)
+// padded rows; cells of an x window of 4 outputs (whole 16-byte words); pitch
+// of P (`side` rows) and of XC in pairs (an odd number of 16-byte words); rows
+// of XC (3 spare rows: the last 4-row group reads past the padded rows)
+__host__ __device__ constexpr int odd_words(int pairs) { return ((pairs + 1) / 2) % 2 ? (pairs + 1) / 2 * 2 : (pairs + 1) / 2 * 2 + 2; }
 __host__ __device__ constexpr int conv_pyr(int R, int side) { return side + 2 * R; }
-__host__ __device__ constexpr int conv_nq(int R) { return (2 * R + 1 + 6) / 4; }
-__host__ __device__ constexpr int conv_px(int R, int side) { return ((side + 3) & ~3) + 4 * conv_nq(R); }
-__host__ __device__ constexpr int conv_xp(int side) { return (side + 3) & ~3; }
+__host__ __device__ constexpr int conv_nv(int R) { return (4 + 2 * R + 1) & ~1; }
+__host__ __device__ constexpr int conv_px(int R, int side) { return odd_words((side + 3) / 4 * 4 - 4 + conv_nv(R)); }
+__host__ __device__ constexpr int conv_xp(int side) { return odd_words((side + 3) / 4 * 4); }
 __host__ __device__ constexpr int conv_xr(int R, int side) { return conv_pyr(R, side) + 3; }
-__host__ __device__ constexpr int conv_mx(int R, int side) { return (conv_pyr(R, side) + 3) & ~3; }
+__host__ __device__ constexpr int conv_mx(int R, int side) { return (conv_pyr(R, side) + 1) & ~1; }
 __host__ __device__ constexpr size_t conv_layout_bytes(int R, int side) {
-    return 128 + sizeof(float) * ((size_t)side * side + (size_t)conv_pyr(R, side) * conv_px(R, side) +
-                                  (size_t)conv_xr(R, side) * conv_xp(side)) +
+    return 128 + sizeof(float) * (size_t)2 * side * side +
+           sizeof(float2) * ((size_t)side * conv_px(R, side) + (size_t)conv_xr(R, side) * conv_xp(side)) +
            sizeof(int) * (size_t)(conv_mx(R, side) + conv_pyr(R, side));
 }
 template <int R, int SIDE>
 struct ConvXYLayout {
     static constexpr int PYR = conv_pyr(R, SIDE);
-    static constexpr int NQ = conv_nq(R);
-    static constexpr int PX = conv_px(R, SIDE);              // room for the last group's window
+    static constexpr int NV = conv_nv(R);
+    static constexpr int PX = conv_px(R, SIDE);
     static constexpr int XP = conv_xp(SIDE);
-    static constexpr int XR = conv_xr(R, SIDE);              // the last 4-row group reads 3 rows past PYR
-    static constexpr int MX = conv_mx(R, SIDE);               // x map entries: whole 4-cell staging groups
-    static constexpr size_t raw = 128;                        // after the barrier
-    static constexpr size_t P = raw + sizeof(float) * SIDE * SIDE;
-    static constexpr size_t XC = P + sizeof(float) * PYR * PX;
-    static constexpr size_t maps = XC + sizeof(float) * XR * XP;
+    static constexpr int XR = conv_xr(R, SIDE);
+    static constexpr int MX = conv_mx(R, SIDE);               // x map entries: whole pairs of cells
+    static constexpr size_t raw = 128;                        // after the barrier: two planes
+    static constexpr size_t P = raw + sizeof(float) * 2 * SIDE * SIDE;
+    static constexpr size_t XC = P + sizeof(float2) * SIDE * PX;
+    static constexpr size_t maps = XC + sizeof(float2) * XR * XP;
     static constexpr size_t bytes = maps + sizeof(int) * (MX + PYR);
     static_assert(bytes == conv_layout_bytes(R, SIDE), "one definition of the layout");
+    static_assert(PX >= MX && P % 16 == 0 && XC % 16 == 0 && maps % 8 == 0, "staged cells and 16-byte words fit");
 };
 
 // Dynamic shared memory of the running launch: the plane kernels refuse to
@@ -137,54 +153,64 @@ __device__ __forceinline__ unsigned dyn_smem_bytes() {
     return r;
 }
 
+// Two FP32 numbers in a 64-bit register, and the FMA rounded for each.
+using Pair = unsigned long long;
+__device__ __forceinline__ Pair make_pair(float lo, float hi) {
+    Pair r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void split_pair(Pair p, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ Pair fma_pair(Pair a, Pair b, Pair c) {
+    Pair r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 __device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
-// raw plane (old layout) -> padded grid P (new layout): a thread per group of
-// four padded cells of a row (16-byte stores; the map has -1 past the row's
-// end, so a group's extra cells take the fill).  Rows outside the old box are
-// not staged: the x pass writes their result directly.
-template <int NT, int PX, class T>
-__device__ __forceinline__ void stage_plane(const T* raw, float* P, const int* mapx, const int* mapy, int PXa, int PYa,
-                                            int onx, float fill, int t) {
-    const int ngp = (PXa + 3) >> 2;
-    const Div16 dg(ngp);
-    for (int j = t; j < PYa * ngp; j += NT) {
-        const int yp = dg(j), xp0 = 4 * (j - yp * ngp);
-        const int my = mapy[yp];
-        if (my < 0) continue;
-        const T* rrow = raw + my * onx;
-        float v[4];
+// raw planes (old layout, the second one PITCH elements on) -> grid P of pairs
+// (the old rows, their columns in the new layout): a warp per row, a lane per
+// two cells (one 16-byte store).  The cells' places in an old row (ix) and
+// whether they and the planes exist (bit 0, 1: the first cell's planes, 2, 3:
+// the second's; else the fill) are the same for all rows of the pair, so a
+// row is loads, selects and a store without a branch.
+template <int NT, int PX, int PITCH, int NL, class T>
+__device__ __forceinline__ void stage_planes(const T* raw, Pair* P, const int2 (&ix)[NL], const unsigned (&in)[NL],
+                                             int PXa, int onx, int ony, float fill, int t) {
+    const int lane = t & 31;
+    for (int y = t >> 5; y < ony; y += NT / 32) {
+        const T* row = raw + y * onx;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int mx = mapx[xp0 + u];
-            v[u] = mx >= 0 ? to_f32(rrow[mx]) : fill;
+        for (int q = 0; q < NL; ++q) {
+            const int xp0 = 2 * (lane + 32 * q);
+            const float a0 = to_f32(row[ix[q].x]), a1 = to_f32(row[ix[q].x + PITCH]);
+            const float b0 = to_f32(row[ix[q].y]), b1 = to_f32(row[ix[q].y + PITCH]);
+            if (xp0 < PXa)
+                *reinterpret_cast<float4*>(P + y * PX + xp0) =
+                    make_float4(in[q] & 1u ? a0 : fill, in[q] & 2u ? a1 : fill, in[q] & 4u ? b0 : fill,
+                                in[q] & 8u ? b1 : fill);
         }
-        *reinterpret_cast<float4*>(P + yp * PX + xp0) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// The plane of item `item` in the box's previous layout: source address and
-// bytes (0 when the new plane lies outside the old box).
-__device__ __forceinline__ void conv_source(const StepBuffers& B, int2 it, const float** src, uint32_t* bytes) {
-    const Box nb = B.cur[it.x], ob = B.prev[it.x];
-    const int ozl = pmod(nb.oz + it.y - ob.oz, B.dom.nz);
-    const int ps = plane_stride(ob.nx, ob.ny);
-    const long long e = ob.off + (long long)(ozl < ob.nz ? ozl : 0) * ps;
-    *src = reinterpret_cast<const float*>(reinterpret_cast<const char*>(B.X) + e * state_bytes(B));
-    *bytes = ozl < ob.nz ? (uint32_t)(ps * state_bytes(B)) : 0u;
-}
+// CTAs per SM the register budget is sized for (shared memory allows them)
+__host__ __device__ constexpr int conv_min_blocks(int side) { return side <= 32 ? 6 : side <= 40 ? 4 : side <= 48 ? 3 : 2; }
 
 template <int R, int SIDE, int NT, bool GRP>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, conv_min_blocks(SIDE))
 p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
     constexpr int W = 2 * R + 1;
     using LY = ConvXYLayout<R, SIDE>;
+    constexpr int NL = (LY::MX + 63) / 64;                  // pairs of cells per lane of a padded row
     extern __shared__ __align__(128) unsigned char smc[];   // ConvXYLayout::bytes
     uint64_t* bar = reinterpret_cast<uint64_t*>(smc);
     float* const raw = reinterpret_cast<float*>(smc + LY::raw);
-    float* const P = reinterpret_cast<float*>(smc + LY::P);
-    float* const XC = reinterpret_cast<float*>(smc + LY::XC);
+    Pair* const P = reinterpret_cast<Pair*>(smc + LY::P);
+    Pair* const XC = reinterpret_cast<Pair*>(smc + LY::XC);
     int* const mapx = reinterpret_cast<int*>(smc + LY::maps);
     int* const mapy = mapx + LY::MX;
     __shared__ int s_flag;
@@ -203,34 +229,41 @@ p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
     __syncthreads();
     if (s_flag) return;
     const Domain D1 = B1.dom;
-    float g[W];
+    Pair gh[R + 1];                                     // the taps are symmetric to the bit
 #pragma unroll
-    for (int k = 0; k < W; ++k) g[k] = taps.g[k];
+    for (int k = 0; k <= R; ++k) gh[k] = make_pair(taps.g[k], taps.g[k]);
+    auto g = [&](int k) { return gh[k <= R ? k : 2 * R - k]; };
     const int n_items = GRP ? group_scan(grp, kItemSlabs, tier, true, s_gb) : B1.st->n_slabs[tier];
     const int2* items = GRP ? nullptr : B1.slab_items + B1.st->slab_base[tier];
     uint32_t phase = 0;
-    bool pending = false;
-    // bulk copy of plane z of box it.x in its previous layout into raw (none
-    // when the plane lies outside the old box)
-    auto fetch = [&](const StepBuffers& Bx, int2 itx, int z) {
-        const float* src;
-        uint32_t bytes;
-        conv_source(Bx, make_int2(itx.x, z), &src, &bytes);
-        if (bytes) {
-            if (t == 0) {
-                fence_async_smem();                     // earlier generic accesses to raw come first
-                mbar_expect(bar, bytes);
-                bulk_load(raw, src, bytes, bar);
-            }
-            pending = true;
+    unsigned pending = 0;                               // bit k: plane k of the next pair is in flight
+    // bulk copies of planes z and z + 1 (below z1) of a box in its previous
+    // layout into raw (none of a plane outside the old box); ozl0: the old
+    // box's plane at the new box's plane 0, cyclically
+    auto fetch = [&](const StepBuffers& Bx, const Box& ob, int ozl0, int z, int z1) {
+        const int nz = Bx.dom.nz;
+        int o0 = ozl0 + z, o1 = o0 + 1;
+        if (o0 >= nz) o0 -= nz;
+        if (o1 >= nz) o1 -= nz;
+        pending = (o0 < ob.nz ? 1u : 0u) | (z + 1 < z1 && o1 < ob.nz ? 2u : 0u);
+        if (pending && t == 0) {
+            const int sb = state_bytes(Bx), ps = plane_stride(ob.nx, ob.ny);
+            const uint32_t bytes = (uint32_t)(ps * sb);
+            const char* src = reinterpret_cast<const char*>(Bx.X) + ob.off * sb;
+            fence_async_smem();                         // earlier generic accesses to raw come first
+            mbar_expect(bar, pending == 3u ? 2u * bytes : bytes);
+            if (pending & 1u) bulk_load(raw, src + (size_t)o0 * bytes, bytes, bar);
+            if (pending & 2u) bulk_load(raw + SIDE * SIDE, src + (size_t)o1 * bytes, bytes, bar);
         }
     };
-    if (blockIdx.x < n_items) {                         // the first item's first plane
-        int lf;
-        const StepBuffers& Bf = member<GRP>(B1, grp, s_gb, blockIdx.x, lf);
-        const int2 itf = list_item<GRP>(Bf, items, kItemSlabs, tier, blockIdx.x, lf);
-        fetch(Bf, itf, itf.y);
-    }
+    auto fetch_item = [&](int i) {                      // an item's first planes
+        int l;
+        const StepBuffers& Bx = member<GRP>(B1, grp, s_gb, i, l);
+        const int2 itx = list_item<GRP>(Bx, items, kItemSlabs, tier, i, l);
+        const Box nb = Bx.cur[itx.x], ob = Bx.prev[itx.x];
+        fetch(Bx, ob, wrap_near(nb.oz - ob.oz, Bx.dom.nz), itx.y, min(itx.y + Bx.slab, nb.nz));
+    };
+    if (blockIdx.x < n_items) fetch_item(blockIdx.x);
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         int local;
         const StepBuffers& B = member<GRP>(B1, grp, s_gb, item, local);
@@ -263,8 +296,23 @@ p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
             if (isx) mapx[ip] = v; else mapy[ip] = v;
         }
         __syncthreads();                                    // the maps are published
-        for (int z = z0; z < z1; ++z) {
-            const bool have = pending;
+        int2 ix[NL];                                        // the staging map of this lane's cells
+        unsigned in_x[NL];
+#pragma unroll
+        for (int q = 0; q < NL; ++q) {
+            const int xp0 = 2 * ((t & 31) + 32 * q);
+            const int2 m = xp0 < PXa ? *reinterpret_cast<const int2*>(mapx + xp0) : make_int2(-1, -1);
+            ix[q] = make_int2(max(m.x, 0), max(m.y, 0));
+            in_x[q] = (m.x >= 0 ? 3u : 0u) | (m.y >= 0 ? 12u : 0u);
+        }
+        const int ozl0 = wrap_near(nb.oz - ob.oz, D.nz);
+        const int ps = plane_stride(nx, ny);
+        const int ngx = (nx + 3) >> 2, ngy = (ny + 3) >> 2;
+        Pair cfill = 0;                                     // the x chain over -eps
+#pragma unroll
+        for (int k = 0; k < W; ++k) cfill = fma_pair(g(k), make_pair(-D.eps, -D.eps), cfill);
+        for (int z = z0; z < z1; z += 2) {
+            const unsigned have = pending;
             bool ok = true;
             if (pending) {
                 ok = mbar_wait(bar, phase, B.wait_limit);
@@ -279,76 +327,83 @@ p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
                 __syncthreads();
                 return;
             }
-            pending = false;
-            // stage: raw (old layout, FP32 or BF16) -> P (new layout), warp per padded row
+            pending = 0;
+            // stage: raw (old layout, FP32 or BF16) -> P (new layout)
             if (have) {
-                if (B.bf16) stage_plane<NT, LY::PX>(reinterpret_cast<const __nv_bfloat16*>(raw), P, mapx, mapy, PXa, PYa,
-                                                    ob.nx, -D.eps, t);
-                else stage_plane<NT, LY::PX>(raw, P, mapx, mapy, PXa, PYa, ob.nx, -D.eps, t);
+                unsigned in[NL];
+#pragma unroll
+                for (int q = 0; q < NL; ++q) in[q] = in_x[q] & (have * 5u);
+                if (B.bf16)
+                    stage_planes<NT, LY::PX, 2 * SIDE * SIDE>(reinterpret_cast<const __nv_bfloat16*>(raw), P, ix, in, PXa,
+                                                              ob.nx, ob.ny, -D.eps, t);
+                else
+                    stage_planes<NT, LY::PX, SIDE * SIDE>(raw, P, ix, in, PXa, ob.nx, ob.ny, -D.eps, t);
             }
-            __syncthreads();                                // raw is free: fetch the next plane
-            if (z + 1 < z1) {
-                fetch(B, it, z + 1);
-            } else if (item + (int)gridDim.x < n_items) {
-                const int nxt = item + gridDim.x;
-                int ln;
-                const StepBuffers& Bn = member<GRP>(B1, grp, s_gb, nxt, ln);
-                const int2 itn = list_item<GRP>(Bn, items, kItemSlabs, tier, nxt, ln);
-                fetch(Bn, itn, itn.y);
-            }
-            // x pass: (padded row, group of 4 outputs)
-            const int ngx = (nx + 3) >> 2;
+            __syncthreads();                                // raw is free: fetch the next planes
+            if (z + 2 < z1) fetch(B, ob, ozl0, z + 2, z1);
+            else if (item + (int)gridDim.x < n_items) fetch_item(item + gridDim.x);
+            // x pass: (group of 4 outputs, padded row), lanes along the rows
             {
-                const Div16 dgx(ngx);
-                float cfill = 0.0f;
-    #pragma unroll
-                for (int k = 0; k < W; ++k) cfill = fmaf(g[k], -D.eps, cfill);
+                const Div16 dpy(PYa);
                 for (int j = t; j < PYa * ngx; j += NT) {
-                    const int yp = dgx(j), x0 = 4 * (j - yp * ngx);
-                    if (!have || mapy[yp] < 0) {                // a fill row: the chain over -eps, unstaged
-                        *reinterpret_cast<float4*>(XC + yp * LY::XP + x0) = make_float4(cfill, cfill, cfill, cfill);
+                    const int gx = dpy(j), yp = j - gx * PYa;
+                    ulonglong2* const out = reinterpret_cast<ulonglong2*>(XC + yp * LY::XP + 4 * gx);
+                    const int my = mapy[yp];
+                    if (!have || my < 0) {                      // a fill row: the chain over -eps
+                        out[0] = out[1] = make_ulonglong2(cfill, cfill);
                         continue;
                     }
-                    const float4* r4 = reinterpret_cast<const float4*>(P + yp * LY::PX + x0);
-                    float v[4 * LY::NQ];
-    #pragma unroll
-                    for (int q = 0; q < LY::NQ; ++q) {
-                        const float4 a = r4[q];
-                        v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
+                    const ulonglong2* r = reinterpret_cast<const ulonglong2*>(P + my * LY::PX + 4 * gx);
+                    Pair v[LY::NV];
+#pragma unroll
+                    for (int q = 0; q < LY::NV / 2; ++q) {
+                        const ulonglong2 a = r[q];
+                        v[2 * q] = a.x;
+                        v[2 * q + 1] = a.y;
                     }
-                    float o[4];
-    #pragma unroll
+                    Pair o[4];
+#pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        float acc = 0.0f;
-    #pragma unroll
-                        for (int k = 0; k < W; ++k) acc = fmaf(g[k], v[u + k], acc);
+                        Pair acc = 0;
+#pragma unroll
+                        for (int k = 0; k < W; ++k) acc = fma_pair(g(k), v[u + k], acc);
                         o[u] = acc;
                     }
-                    *reinterpret_cast<float4*>(XC + yp * LY::XP + x0) = make_float4(o[0], o[1], o[2], o[3]);
+                    out[0] = make_ulonglong2(o[0], o[1]);
+                    out[1] = make_ulonglong2(o[2], o[3]);
                 }
             }
             __syncthreads();
             // y pass: (group of 4 rows, column), lanes along x
             {
-                float* dst = B.Z + nb.off + (long long)z * plane_stride(nx, ny);
-                const int ngy = (ny + 3) >> 2;
+                float* const dst = B.Z + nb.off + (long long)z * ps;
+                float* const dst2 = dst + ps;
+                const bool two = z + 1 < z1;
                 const Div16 dnx(nx);
                 for (int j = t; j < ngy * nx; j += NT) {
                     const int gy = dnx(j), x = j - gy * nx, y0 = 4 * gy;
-                    const float* col = XC + y0 * LY::XP + x;
-                    float v[W + 3];
-    #pragma unroll
+                    const Pair* col = XC + y0 * LY::XP + x;
+                    Pair v[W + 3];
+#pragma unroll
                     for (int k = 0; k < W + 3; ++k) v[k] = col[k * LY::XP];
-    #pragma unroll
+                    unsigned o = (unsigned)(y0 * nx + x);
+                    const int left = ny - y0;
+#pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        float acc = 0.0f;
-    #pragma unroll
-                        for (int k = 0; k < W; ++k) acc = fmaf(g[k], v[u + k], acc);
-                        if (y0 + u < ny) dst[(y0 + u) * nx + x] = acc;
+                        Pair acc = 0;
+#pragma unroll
+                        for (int k = 0; k < W; ++k) acc = fma_pair(g(k), v[u + k], acc);
+                        float lo, hi;
+                        split_pair(acc, lo, hi);
+                        if (u < left) {
+                            dst[o] = lo;
+                            if (two) dst2[o] = hi;
+                        }
+                        o += nx;
                     }
                 }
             }
-            __syncthreads();                                // XC is free
+            // the next pair's x pass, the next writer of XC, is two barriers away
         }
     }
 }

@@ -169,3 +169,25 @@ def test_physics_z_pass_against_the_oracle(L, kind, dims, G, bf16):
     for g in phip:
         want = O.predict(ref.grains[g], shape, taps, 7.0, ph, 1.0)
         assert np.max(np.abs(phip[g] - want)) <= 3e-5, g
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,G", [
+    ((96, 90, 84), 20),              # sides over 40 and over 48: the larger plane grids
+    ((33, 70, 41), 12),              # odd numbers of planes, boxes across full axes of odd length
+    ((24, 24, 24), 30),              # small boxes
+])
+def test_ideal_convolution_against_the_oracle(L, dims, G, bf16):
+    """phi_p of the third step (boxes moved since the state was stored) within the parity tests' 2e-5."""
+    from oracle import lsgg_oracle as O
+    from tests.parity import oracle_from_gpu
+    shape = (dims[2], dims[1], dims[0])
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(21, G, dims),
+                          storage=L.STORAGE_BF16 if bf16 else L.STORAGE_FP32) as ms:
+        ms.step(2, 1.0)
+        ms.sync()
+        ref = oracle_from_gpu(shape, ms.boxes(), ms.phi())
+        _, (phip, *_rest) = ms.debug_step(1.0)
+    taps = O.heat_kernel_taps(1.0, 5)
+    for g in phip:
+        assert np.max(np.abs(phip[g] - O.predict(ref.grains[g], shape, taps, 7.0))) <= 2e-5, g
