@@ -191,3 +191,36 @@ def test_ideal_convolution_against_the_oracle(L, dims, G, bf16):
     taps = O.heat_kernel_taps(1.0, 5)
     for g in phip:
         assert np.max(np.abs(phip[g] - O.predict(ref.grains[g], shape, taps, 7.0))) <= 2e-5, g
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,G", [
+    ((26, 28, 140), 9),              # columns of every length up to a hundred, long ones past the register form
+    ((60, 58, 62), 45),
+    ((24, 25, 23), 4),               # periodic on every axis
+    ((130, 20, 22), 5),              # boxes wider than the shared-memory plane grids
+])
+def test_reinitialisation_of_the_step_s_own_phi_c(L, dims, G, bf16):
+    """phi after the step against the oracle's re-initialisation of the step's phi_c: the same FP32 inputs, at most
+    six roundings of values up to 7 and the reciprocal square root of the distance (2 ulp): 1e-5; in BF16 the
+    stored value's rounding, 2^-8 of it, on top."""
+    from oracle import lsgg_oracle as O
+    shape = (dims[2], dims[1], dims[0])
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(23, G, dims),
+                          storage=L.STORAGE_BF16 if bf16 else L.STORAGE_FP32) as ms:
+        ms.step(1, 1.0)
+        ms.sync()
+        boxes, (_, _, _, phic, phin) = ms.debug_step(1.0)
+        phi = ms.phi()
+        new = ms.boxes()
+    for g in phin:
+        b = boxes[g]
+        full = tuple(int(b[6 - a]) == shape[a] for a in range(3))
+        want = O.redistance(phic[g].astype(np.float64), full, 7.0, (0, 1, 2))
+        assert np.array_equal(phin[g] > 0, phic[g] > 0)
+        assert np.max(np.abs(phin[g] - want)) <= 1e-5, g
+        if new[g, 0]:                                # the stored state: the same values on the new box
+            was = O.Grain(g, (int(b[3]), int(b[2]), int(b[1])), phin[g].astype(np.float64))
+            box = O.Grain(g, tuple(int(v) for v in new[g, 3:0:-1]), np.zeros(tuple(int(v) for v in new[g, 6:3:-1])))
+            kept = O.sample(was, O.box_positions(box, shape), shape, -7.0)[0]
+            assert np.all(np.abs(phi[g] - kept) <= (2.0 ** -8 * np.abs(kept) if bf16 else 0.0)), g
