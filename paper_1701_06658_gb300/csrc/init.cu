@@ -821,42 +821,64 @@ __global__ void k_label_occupancy(Domain D, const int* __restrict__ labels, unsi
 // holding every occupied position -- the complement of the longest run of
 // empty positions, the first such run (smallest start) on ties -- grown by
 // the halo and capped at the axis; no cell: extinct.
-__global__ void k_label_boxes(Domain D, int G, const unsigned* __restrict__ occ, int words, Box* __restrict__ cur) {
+// A warp per grain: its lanes look for the starts of empty runs and follow
+// them word by word (one thread per grain, bit by bit, took 0.6 ms on a
+// 149 x 97 x 61 domain on GB300).
+__global__ void __launch_bounds__(128)
+k_label_boxes(Domain D, int G, const unsigned* __restrict__ occ, int words, Box* __restrict__ cur) {
     const int N[3] = {D.nx, D.ny, D.nz};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < G; i += gridDim.x * blockDim.x) {
-        const unsigned* ox = occ + ((long long)i * 3) * words;
-        bool any = false;
-        for (int w = 0; w < words; ++w) any = any || ox[w] != 0u;
-        Box b{};
-        if (!any) {
-            cur[i] = b;
-            continue;
-        }
-        int o[3], n[3];
-        for (int a = 0; a < 3; ++a) {
-            const int na = N[a];
-            if (na == 1) { o[a] = 0; n[a] = 1; continue; }
-            const unsigned* bits = occ + ((long long)i * 3 + a) * words;
-            auto at = [&](int p) { return (bits[p >> 5] >> (p & 31)) & 1u; };
-            int best_start = 0, best_len = -1;
-            for (int p = 0; p < na; ++p) {
-                if (at(p) || !at(p == 0 ? na - 1 : p - 1)) continue;   // not the first empty position of a run
-                int len = 0;
-                while (len < na && !at((p + len) % na)) ++len;
-                if (len > best_len) { best_start = p; best_len = len; }
-            }
-            int start = 0, length = na;                            // every position held
-            if (best_len > 0) {
-                start = (best_start + best_len) % na;
-                length = na - best_len;
-            }
-            n[a] = length + 2 * D.halo < na ? length + 2 * D.halo : na;
-            o[a] = pmod(start - D.halo, na);
-        }
-        b.ox = o[0]; b.oy = o[1]; b.oz = o[2];
-        b.nx = n[0]; b.ny = n[1]; b.nz = n[2];
-        cur[i] = b;
+    const int lane = threadIdx.x & 31;
+    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= G) return;                                       // uniform across the warp
+    const unsigned* ox = occ + ((long long)i * 3) * words;
+    bool any = false;
+    for (int w = lane; w < words; w += 32) any = any || ox[w] != 0u;
+    Box b{};
+    if (!__any_sync(0xffffffffu, any)) {
+        if (lane == 0) cur[i] = b;
+        return;
     }
+    int o[3], n[3];
+    for (int a = 0; a < 3; ++a) {
+        const int na = N[a];
+        if (na == 1) { o[a] = 0; n[a] = 1; continue; }
+        const unsigned* bits = occ + ((long long)i * 3 + a) * words;
+        auto at = [&](int p) { return (bits[p >> 5] >> (p & 31)) & 1u; };
+        // the longest run, the smallest start on ties, as one key
+        unsigned long long best = 0;
+        for (int p = lane; p < na; p += 32) {
+            if (at(p) || !at(p == 0 ? na - 1 : p - 1)) continue;   // not the first empty position of a run
+            int len = 0;
+            for (int q = p; len < na;) {                      // empty positions from p on, a word at a time
+                const int room = min(32 - (q & 31), na - q);  // positions of this word
+                unsigned m = bits[q >> 5] >> (q & 31);
+                if (room < 32) m |= 1u << room;               // ends the search at the word's (axis') end
+                const int free_ = m ? __ffs(m) - 1 : 32;
+                len += free_;
+                if (free_ < room) break;
+                q = q + room >= na ? 0 : q + room;
+            }
+            len = min(len, na);
+            const unsigned long long key = ((unsigned long long)len << 32) | (0xffffffffu - (unsigned)p);
+            best = key > best ? key : best;
+        }
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, best, k);
+            best = v > best ? v : best;
+        }
+        int start = 0, length = na;                           // every position held
+        if (best) {
+            const int best_len = (int)(best >> 32), best_start = (int)(0xffffffffu - (unsigned)(best & 0xffffffffu));
+            start = (best_start + best_len) % na;
+            length = na - best_len;
+        }
+        n[a] = length + 2 * D.halo < na ? length + 2 * D.halo : na;
+        o[a] = pmod(start - D.halo, na);
+    }
+    b.ox = o[0]; b.oy = o[1]; b.oz = o[2];
+    b.nx = n[0]; b.ny = n[1]; b.nz = n[2];
+    if (lane == 0) cur[i] = b;
 }
 
 // The starting function before the re-initialisation: +1/2 on the grain's
@@ -869,7 +891,7 @@ __global__ void k_label_phi(Domain D, const Box* __restrict__ cur, const int* __
     const int ps = plane_stride(b.nx, b.ny);
     const int A = b.nx * b.ny;
     const long long n = (long long)A * b.nz;
-    for (long long k = threadIdx.x; k < n; k += blockDim.x) {
+    for (long long k = blockIdx.y * blockDim.x + threadIdx.x; k < n; k += gridDim.y * blockDim.x) {
         const int z = (int)(k / A), rem = (int)(k - (long long)z * A);
         const int y = rem / b.nx, x = rem - y * b.nx;
         const long long g = ((long long)pmod(b.oz + z, D.nz) * D.ny + pmod(b.oy + y, D.ny)) * D.nx + pmod(b.ox + x, D.nx);
@@ -885,12 +907,12 @@ cudaError_t launch_label_boxes(const Domain& D, int G, const int* d_labels, unsi
     long long gs = (ncell + 255) / 256;
     if (gs > 65535 * 8) gs = 65535 * 8;
     k_label_occupancy<<<(int)gs, 256, 0, s>>>(D, d_labels, d_occ, words);
-    k_label_boxes<<<(G + 127) / 128, 128, 0, s>>>(D, G, d_occ, words, d_cur);
+    k_label_boxes<<<(G + 3) / 4, 128, 0, s>>>(D, G, d_occ, words, d_cur);
     return cudaGetLastError();
 }
 
 cudaError_t launch_label_phi(const Domain& D, int G, const Box* d_cur, const int* d_labels, float* Z, cudaStream_t s) {
-    k_label_phi<<<G, 256, 0, s>>>(D, d_cur, d_labels, Z);
+    k_label_phi<<<dim3(G, 8), 256, 0, s>>>(D, d_cur, d_labels, Z);
     return cudaGetLastError();
 }
 

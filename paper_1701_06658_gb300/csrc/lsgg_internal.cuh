@@ -34,6 +34,7 @@ constexpr int kMaxTaps = 2 * kMaxRadius + 1;
 constexpr int kNumClasses = 5;          // box side <= 32, 40, 48, 64, larger (global scratch)
 constexpr int kRedistReach = 6;         // taxicab steps below eps = 7 (exact fixed point)
 constexpr int kTiers = 5;               // pass path: boxes with x, y sides <= 32, <= 40, <= 48, <= 64, larger
+constexpr int kFewBoxes = 2048;         // up to this many boxes, kernels of a CTA per box take a cluster per box
 constexpr int kPassChunk = 256;         // columns per column item of the pass path
 constexpr int kSlab = 8;                // planes per slab item of the pass path (default; autotuned)
 constexpr int kMinSlab = 4;             // the smallest slab the autotuner tries (sizes the slab item list)

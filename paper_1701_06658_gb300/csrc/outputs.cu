@@ -1,27 +1,26 @@
 // Outputs of a microstructure.
 //
-//   k_volumes   V_i = sum_x H(phi_i(x)), H(phi) = clamp(phi + 1/2, 0, 1): one CTA
-//               per box over the state's own layout (`prev`), 16-byte loads,
-//               four in flight per thread.  Each thread sums its cells in
-//               fixed point (H in units of 2^-28 is an integer, exactly for
-//               every |phi| >= 2^-5 and to 2^-29 below, so the 64-bit sum is
-//               exact); the threads' partials are merged in FP64 with
-//               compensated (TwoSum) additions in a fixed tree order.  For a
-//               box of fewer than 2^25 cells every partial sum is an integer
-//               multiple of 2^-28 below 2^25, exact in FP64, so the result is
-//               the exact sum whatever the cells' order; larger boxes keep the
-//               compensated sum's rounding, the same on every run.
+//   k_volumes   V_i = sum_x H(phi_i(x)), H(phi) = clamp(phi + 1/2, 0, 1): a
+//               cluster of CTAs per box over the state's own layout (`prev`),
+//               16-byte loads, four in flight per thread.  The cells are summed
+//               in fixed point (H in units of 2^-28 is an integer, exactly for
+//               every |phi| >= 2^-5 and to 2^-29 below), so that the 64-bit sum
+//               is exact whatever the cells' order, and the volume is that sum
+//               rounded once to FP64 (below 2^25 cells it needs no rounding).
 //   k_owner_*   owner(x) = argmax_i phi_i(x) over boxes covering x, lowest id on
 //               ties (64-bit atomicMax of (phi, -id) keys), -1 where uncovered.
 //   k_remap     the state phi (stored in the `prev` layout) resampled on the
 //               current boxes with -eps where the old box did not reach: the
 //               grain functions as they enter the next step (Sec. 3.1 box update).
 #include <algorithm>
+#include <cooperative_groups.h>
 
 #include "lsgg_internal.cuh"
 #include "../../include/lsgg.h"
 
 namespace lsgg {
+
+namespace cg = cooperative_groups;
 
 __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
     s = __dadd_rn(a, b);
@@ -57,15 +56,15 @@ constexpr int kVolLoads = 4;     // 16-byte loads in flight per thread
 // the same in any order.  I: the index type (32-bit divisions whenever the
 // items fit).
 template <class I>
-__device__ __forceinline__ long long volume_walk(const float* base, int A, int ps, int nz) {
+__device__ __forceinline__ long long volume_walk(const float* base, int A, int ps, int nz, int part, int parts) {
     const I nq = (I)((A + 3) >> 2);
     const I items = nq * (I)nz;
     long long acc = 0;
-    for (I i0 = threadIdx.x; i0 < items; i0 += (I)kVolLoads * blockDim.x) {
+    for (I i0 = (I)part * blockDim.x + threadIdx.x; i0 < items; i0 += (I)(kVolLoads * parts) * blockDim.x) {
         float v[kVolLoads][4];
 #pragma unroll
         for (int k = 0; k < kVolLoads; ++k) {
-            const I it = i0 + (I)k * blockDim.x;
+            const I it = i0 + (I)(k * parts) * blockDim.x;
             const I z = it < items ? it / nq : 0;
             const int q = it < items ? 4 * (int)(it - z * nq) : 0;
             const float* pl = base + (long long)z * ps;
@@ -88,35 +87,42 @@ __device__ __forceinline__ long long volume_walk(const float* base, int A, int p
 // The state lives in the `prev` layout; a cell of the prev box outside the
 // current box is at least halo + 1 cells from every positive cell, so its
 // phi <= -halo and H = 0: summing the prev box is summing the current box.
-__global__ void __launch_bounds__(256)
+// One CTA per box leaves a box far larger than the others (a grown grain: 10^6
+// cells) on one SM at the end of the launch: 160^3 lognormal 700 us on GB300,
+// 138 us with eight CTAs a box, 64^3 / 50 grains 32 and 13 us.  With many boxes
+// the clusters cost more than they balance (256^3 / 5000: 178 us with one CTA a
+// box, 291 with eight).
+template <int CL>                // CTAs per box: a thread-block cluster
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(256)
 k_volumes(Domain D, const Box* __restrict__ cur, const Box* __restrict__ prev, const float* __restrict__ X,
           double* __restrict__ out) {
-    __shared__ double s_s[256], s_c[256];
-    const int b = blockIdx.x;
-    constexpr int kOne = 1 << 28;
+    __shared__ unsigned long long s_sum;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int part = (int)cluster.block_rank();
+    const int b = blockIdx.x / CL;
+    if (threadIdx.x == 0) s_sum = 0;
+    cluster.sync();                                  // the first CTA's sum is clear before any addition
     long long acc = 0;
     if (cur[b].nx > 0) {
         const Box ob = prev[b];
         const int A = ob.nx * ob.ny, ps = plane_stride(ob.nx, ob.ny);
-        if ((long long)((A + 3) >> 2) * ob.nz < (1LL << 31) - 4LL * kVolLoads * 256)
-            acc = volume_walk<unsigned>(X + ob.off, A, ps, ob.nz);
+        if ((long long)((A + 3) >> 2) * ob.nz < (1LL << 31) - 4LL * kVolLoads * CL * 256)
+            acc = volume_walk<unsigned>(X + ob.off, A, ps, ob.nz, part, CL);
         else
-            acc = volume_walk<long long>(X + ob.off, A, ps, ob.nz);
+            acc = volume_walk<long long>(X + ob.off, A, ps, ob.nz, part, CL);
     }
-    s_s[threadIdx.x] = (double)acc / (double)kOne;   // exact: acc < 2^53
-    s_c[threadIdx.x] = 0.0;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < (unsigned)o) {
-            double t, e;
-            two_sum(s_s[threadIdx.x], s_s[threadIdx.x + o], t, e);
-            s_s[threadIdx.x] = t;
-            s_c[threadIdx.x] = __dadd_rn(__dadd_rn(s_c[threadIdx.x], s_c[threadIdx.x + o]), e);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[b] = __dadd_rn(s_s[0], s_c[0]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0 && acc) atomicAdd(cluster.map_shared_rank(&s_sum, 0), (unsigned long long)acc);
+    cluster.sync();
+    constexpr double kOne = 268435456.0;             // 2^28
+    if (part == 0 && threadIdx.x == 0) out[b] = (double)s_sum / kOne;
 }
+
+// CTAs a box's cells are spread over (grid y) with few boxes: one CTA per box
+// would leave the largest box on one SM (owner map of a 160^3 lognormal run 4.3
+// ms on GB300, 0.7 with eight).
+static int box_parts(int G) { return G <= kFewBoxes ? 8 : 1; }
 
 __global__ void __launch_bounds__(256)
 k_owner_scatter(Domain D, const Box* __restrict__ cur, const Box* __restrict__ prev, const float* __restrict__ X,
@@ -125,15 +131,19 @@ k_owner_scatter(Domain D, const Box* __restrict__ cur, const Box* __restrict__ p
     const Box nb = cur[b];
     if (nb.nx <= 0) return;
     const Box ob = prev[b];
-    const long long A = (long long)nb.nx * nb.ny;
-    const long long n = A * nb.nz;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-        int z = (int)(i / A);
-        int rem = (int)(i - z * A);
-        int y = rem / nb.nx, x = rem - y * nb.nx;
-        float v = state_value(D, nb, ob, X, x, y, z);
-        long long g = ((long long)pmod(nb.oz + z, D.nz) * D.ny + pmod(nb.oy + y, D.ny)) * D.nx + pmod(nb.ox + x, D.nx);
-        atomicMax(&F[g], make_key(v, b));
+    // rows of the box, a warp each; a key that is below the cell's by now
+    // takes no atomic (the cell's only grows)
+    const int rows = nb.ny * nb.nz, lane = threadIdx.x & 31;
+    for (int r = (int)(blockIdx.y * blockDim.x + threadIdx.x) >> 5; r < rows; r += (int)(gridDim.y * blockDim.x) >> 5) {
+        const int z = r / nb.ny, y = r - z * nb.ny;
+        const long long g0 = ((long long)pmod(nb.oz + z, D.nz) * D.ny + pmod(nb.oy + y, D.ny)) * D.nx;
+        for (int x = lane; x < nb.nx; x += 32) {
+            const float v = state_value(D, nb, ob, X, x, y, z);
+            int gx = nb.ox + x;
+            if (gx >= D.nx) gx -= D.nx;
+            const unsigned long long key = make_key(v, b);
+            if (key > *(volatile unsigned long long*)&F[g0 + gx]) atomicMax(&F[g0 + gx], key);
+        }
     }
 }
 
@@ -152,7 +162,7 @@ k_pack_state(Domain D, const Box* __restrict__ cur, const Box* __restrict__ prev
     const Box ob = prev[b];
     const long long A = (long long)nb.nx * nb.ny;
     const long long n = A * nb.nz;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+    for (long long i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
         int z = (int)(i / A);
         int rem = (int)(i - z * A);
         int y = rem / nb.nx, x = rem - y * nb.nx;
@@ -198,7 +208,8 @@ k_unpack_state(const Box* __restrict__ cur, const float* __restrict__ packed, co
 
 cudaError_t launch_volumes(const Domain& D, int G, const Box* cur, const Box* prev, const float* X, double* out,
                            cudaStream_t s) {
-    k_volumes<<<G, 256, 0, s>>>(D, cur, prev, X, out);
+    if (G <= kFewBoxes) k_volumes<8><<<G * 8, 256, 0, s>>>(D, cur, prev, X, out);
+    else k_volumes<1><<<G, 256, 0, s>>>(D, cur, prev, X, out);
     return cudaGetLastError();
 }
 
@@ -207,7 +218,7 @@ cudaError_t launch_owner(const Domain& D, int G, const Box* cur, const Box* prev
     long long n = (long long)D.nx * D.ny * D.nz;
     cudaError_t e = cudaMemsetAsync(F, 0, (size_t)n * 8, s);
     if (e != cudaSuccess) return e;
-    k_owner_scatter<<<G, 256, 0, s>>>(D, cur, prev, X, F);
+    k_owner_scatter<<<dim3(G, box_parts(G)), 256, 0, s>>>(D, cur, prev, X, F);
     int blocks = (int)((n + 255) / 256);
     if (blocks > 65535 * 16) blocks = 65535 * 16;
     k_owner_decode<<<blocks, 256, 0, s>>>(n, F, out);
@@ -229,7 +240,7 @@ cudaError_t launch_step_status(const StepState* st, int* out, cudaStream_t s) {
 
 cudaError_t launch_pack_state(const Domain& D, int G, const Box* cur, const Box* prev, const float* X,
                               const long long* packed_off, float* out, cudaStream_t s) {
-    k_pack_state<<<G, 256, 0, s>>>(D, cur, prev, X, packed_off, out);
+    k_pack_state<<<dim3(G, box_parts(G)), 256, 0, s>>>(D, cur, prev, X, packed_off, out);
     return cudaGetLastError();
 }
 

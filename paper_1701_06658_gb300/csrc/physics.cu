@@ -91,35 +91,41 @@ __device__ __forceinline__ void collect_walk(const int* base, int A, int ps, int
     }
 }
 
-constexpr int kCollectCluster = 4;    // CTAs per box: a thread-block cluster
-
-// A cluster of kCollectCluster CTAs per box: each walks a part of the box's
-// ID-field and enters its ids into the hash in the shared memory of the
-// cluster's first CTA (distributed shared memory), which then does the rest.
-__global__ void __cluster_dims__(kCollectCluster, 1, 1) __launch_bounds__(kCollectThreads)
+// A cluster of CL CTAs per box: each walks a part of the box's
+// ID-field into a hash of its own, then enters the ids it found into the hash
+// of the cluster's first CTA (distributed shared memory), which does the rest.
+// Entering every run of equal ids into the first CTA's hash at once made each
+// probe a remote access: 160^3 lognormal (one box of 10^6 cells) 462 us a step
+// on GB300, 207 us with hashes of their own and eight CTAs a box.
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kCollectThreads)
 k_collect_neighbours(PhysicsDev phys, StepState* st, const Box* __restrict__ prev, const int* __restrict__ IDF,
                      int* __restrict__ tab, int* __restrict__ cnt, float* __restrict__ tw, float* __restrict__ tm) {
     __shared__ int keys[kHashSlots];
     __shared__ int n_keys, overflow;
     cg::cluster_group cluster = cg::this_cluster();
     const int part = (int)cluster.block_rank();
-    const int b = blockIdx.x / kCollectCluster;
+    const int b = blockIdx.x / CL;
     const Box ob = prev[b];
-    if (part == 0) {
-        for (int k = threadIdx.x; k < kHashSlots; k += blockDim.x) keys[k] = -1;
-        if (threadIdx.x == 0) { n_keys = 0; overflow = 0; }
-    }
-    cluster.sync();                                  // the first CTA's hash is clear before any entry
+    for (int k = threadIdx.x; k < kHashSlots; k += blockDim.x) keys[k] = -1;
+    if (threadIdx.x == 0) { n_keys = 0; overflow = 0; }
+    __syncthreads();
     if (ob.nx > 0) {
-        int* const k0 = cluster.map_shared_rank(keys, 0);
-        int* const n0 = cluster.map_shared_rank(&n_keys, 0);
-        int* const o0 = cluster.map_shared_rank(&overflow, 0);
         const int A = ob.nx * ob.ny;
         const int ps = plane_stride(ob.nx, ob.ny);
         if ((long long)((A + 3) >> 2) * ob.nz < (1LL << 31) - 4LL * kCollectLoads * kCollectThreads)
-            collect_walk<unsigned>(IDF + ob.off, A, ps, ob.nz, part, kCollectCluster, k0, n0, o0);
+            collect_walk<unsigned>(IDF + ob.off, A, ps, ob.nz, part, CL, keys, &n_keys, &overflow);
         else
-            collect_walk<long long>(IDF + ob.off, A, ps, ob.nz, part, kCollectCluster, k0, n0, o0);
+            collect_walk<long long>(IDF + ob.off, A, ps, ob.nz, part, CL, keys, &n_keys, &overflow);
+    }
+    cluster.sync();                                  // every CTA's hash is complete
+    if (part != 0) {
+        int* const k0 = cluster.map_shared_rank(keys, 0);
+        int* const n0 = cluster.map_shared_rank(&n_keys, 0);
+        int* const o0 = cluster.map_shared_rank(&overflow, 0);
+        for (int k = threadIdx.x; k < kHashSlots; k += blockDim.x)
+            if (keys[k] >= 0) collect_key(k0, n0, o0, keys[k]);
+        if (threadIdx.x == 0 && overflow) *o0 = 1;
     }
     cluster.sync();                                  // every entry is in; the other CTAs are done
     if (part != 0) return;
@@ -249,14 +255,21 @@ cudaError_t launch_field_neighbours(const StepBuffers& B, const Box* boxes, int 
     return cudaGetLastError();
 }
 
+// CTAs per box with few boxes (whose largest one outlasts the others) and with
+// many: 512^3 / 40 000 grains, step 21.3 ms at one CTA a box, 20.4 at two, 20.7
+// at four (2.2 ms of it this kernel), 21.4 at eight.
+constexpr int kCollectFew = 8, kCollectMany = 2;
+
 cudaError_t launch_collect_neighbours(const StepBuffers& B, const PhysicsDev& phys, cudaStream_t s) {
     if (phys.pool_ent[0]) {
         const cudaError_t e = cudaMemsetAsync(&B.st->pool_used, 0, sizeof(int), s);
         if (e != cudaSuccess) return e;
     }
-    k_collect_neighbours<<<B.n_boxes * kCollectCluster, kCollectThreads, 0, s>>>(phys, B.st, B.prev, B.IDF, const_cast<int*>(phys.nb_tab),
-                                                     const_cast<int*>(phys.nb_cnt), const_cast<float*>(phys.nb_w),
-                                                     const_cast<float*>(phys.nb_m));
+    const bool few = B.n_boxes <= kFewBoxes;
+    (few ? k_collect_neighbours<kCollectFew> : k_collect_neighbours<kCollectMany>)
+        <<<B.n_boxes * (few ? kCollectFew : kCollectMany), kCollectThreads, 0, s>>>(
+            phys, B.st, B.prev, B.IDF, const_cast<int*>(phys.nb_tab), const_cast<int*>(phys.nb_cnt),
+            const_cast<float*>(phys.nb_w), const_cast<float*>(phys.nb_m));
     return cudaGetLastError();
 }
 
