@@ -1176,22 +1176,6 @@ static FieldFn field_fn(int tx, bool ids, bool idf, bool dg) {
 // the whole line equals the 6-step window because no magnitude exceeds
 // eps = 7.
 
-// The scan of a periodic line of n values in shared memory (their magnitudes
-// go in and come out): twice around in each direction.
-__device__ __forceinline__ void scan_line_wrap(float* L, int n, int st) {
-    float f = fabsf(L[0]);
-    for (int j = 1; j < 2 * n; ++j) {
-        const int i = j < n ? j : j - n;
-        f = fminf(fabsf(L[i * st]), f + 1.0f);
-        L[i * st] = f;
-    }
-    for (int j = 2 * n - 2; j >= 0; --j) {
-        const int i = j < n ? j : j - n;
-        f = fminf(L[i * st], f + 1.0f);
-        L[i * st] = f;
-    }
-}
-
 // Segmented min-plus scan of a line held in registers by the LANES
 // consecutive lanes that share it: lane `seg` holds cells [seg * L, seg * L +
 // L) and scans them forward and backward; between the two directions it
@@ -1224,6 +1208,54 @@ __device__ __forceinline__ float with_sign(float d, unsigned m, int j) {
     return __uint_as_float(__float_as_uint(d) | (~(m << (31 - j)) & 0x80000000u));
 }
 
+// The scan of a periodic line of n cells, `nb` of them (from x0 on) this
+// lane's, their magnitudes in r; `line` holds every cell (stride st, signs
+// ignored) and is left with the forward scan.  A line scanned twice around in
+// either direction gives each cell the least of the kRedistReach cells before
+// (behind) it plus their distance, added one at a time, since a value carried
+// further is eps at least: so each lane starts kRedistReach cells ahead of its
+// own.  Bound by the chain of dependent shared-memory reads: one lane scanning
+// the whole line twice around made a step of a 32^3 periodic domain 0.157 ms
+// on GB300, this 0.126.  All lanes of the warp must call.
+template <int L>
+__device__ __forceinline__ void scan_seg_wrap(float* line, int st, int n, int x0, int nb, float (&r)[L]) {
+    float f = 0.0f;
+    if (nb > 0) {
+        int i = pmod(x0 - kRedistReach, n);
+        f = fabsf(line[i * st]);
+#pragma unroll
+        for (int k = 1; k < kRedistReach; ++k) {
+            i = i + 1 == n ? 0 : i + 1;
+            f = fminf(fabsf(line[i * st]), f + 1.0f);
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < L; ++j)
+        if (j < nb) {
+            f = fminf(r[j], f + 1.0f);
+            r[j] = f;
+            line[(x0 + j) * st] = f;
+        }
+    __syncwarp();
+    if (nb > 0) {
+        int i = pmod(x0 + nb - 1 + kRedistReach, n);
+        f = line[i * st];
+#pragma unroll
+        for (int k = 1; k < kRedistReach; ++k) {
+            i = i == 0 ? n - 1 : i - 1;
+            f = fminf(line[i * st], f + 1.0f);
+        }
+    }
+#pragma unroll
+    for (int j = L - 1; j >= 0; --j)
+        if (j < nb) {
+            f = fminf(r[j], f + 1.0f);
+            r[j] = f;
+        }
+    __syncwarp();
+}
+
 // Plane pass of the re-initialisation: a CTA of NT = 4 * SIDE threads takes
 // one (box, slab of kSlab planes) item at a time and walks its planes in z
 // order.  Planes of phi_c stream into a 3-slot shared-memory ring by bulk
@@ -1238,8 +1270,8 @@ __device__ __forceinline__ float with_sign(float d, unsigned m, int j) {
 // for the planar-exact distance; every other cell starts at eps.  The x scan
 // runs in the owner's registers (one carry exchange between the four lanes
 // of a row) and goes with the signs of phi_c to the grid G; thread (c, s) then
-// scans rows [s L, s L + L) of column c the same way and stores plane z.  A
-// full periodic axis takes a serial scan twice around the line by one lane.
+// scans rows [s L, s L + L) of column c the same way and stores plane z.  On a
+// full periodic axis each lane starts its scans kRedistReach cells ahead.
 //
 // The pass is bound by its instructions, so what cannot change is left out:
 // a plane without a positive cell in itself and both neighbours is -eps (the
@@ -1455,14 +1487,11 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
                         rr[j] = (ref >> j) & 1u ? g : eps;
                     }
                     if (!fx) scan_seg_regs<L, LANES>(rr, s, eps);
-                    else {                                  // periodic x: the row twice around, one lane
+                    else {
 #pragma unroll
                         for (int j = 0; j < L; ++j) grow[j] = rr[j];
                         __syncwarp();
-                        if (s == 0 && r < ny) scan_line_wrap(G + r * PG, nx, 1);
-                        __syncwarp();
-#pragma unroll
-                        for (int j = 0; j < L; ++j) rr[j] = grow[j];
+                        scan_seg_wrap<L>(G + r * PG, 1, nx, x0, r < ny ? nbits : 0, rr);
                     }
                     // rows past ny and cells past nx of G are written but never used
 #pragma unroll
@@ -1486,28 +1515,18 @@ p_redist_xy(StepBuffers B1, GroupRef grp, int tier) {
                 const float* const gcol = G + x0 * PG + c;
                 float* dc = dst + x0 * nx + c;
                 const int nrow = c < nx ? min(ny - x0, L) : 0;         // rows of the segment to store
-                float rr[L];
-                if (!fy) {
-                    float sg[L];
+                float sg[L], rr[L];
 #pragma unroll
-                    for (int j = 0; j < L; ++j) {
-                        sg[j] = gcol[j * PG];                          // in bounds; rows past ny are eps
-                        rr[j] = fabsf(sg[j]);
-                    }
-                    scan_seg_regs<L, LANES>(rr, s, eps);
+                for (int j = 0; j < L; ++j) {
+                    sg[j] = gcol[j * PG];                              // in bounds; rows past ny are eps
+                    rr[j] = fabsf(sg[j]);
+                }
+                if (!fy) scan_seg_regs<L, LANES>(rr, s, eps);
+                else scan_seg_wrap<L>(G + c, PG, ny, x0, max(nrow, 0), rr);
 #pragma unroll
-                    for (int j = 0; j < L; ++j) {
-                        if (j < nrow) *dc = copysignf(rr[j], sg[j]);
-                        dc += nx;
-                    }
-                } else {                                    // periodic y: the column twice around, one lane
-                    if (s == 0 && c < nx) scan_line_wrap(G + c, ny, PG);
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < L; ++j) {
-                        if (j < nrow) *dc = Pc[(x0 + j) * nx + c] > 0.0f ? fabsf(gcol[j * PG]) : -fabsf(gcol[j * PG]);
-                        dc += nx;
-                    }
+                for (int j = 0; j < L; ++j) {
+                    if (j < nrow) *dc = copysignf(rr[j], sg[j]);
+                    dc += nx;
                 }
             }
         }
@@ -2014,22 +2033,10 @@ cudaError_t launch_sweep_redist(const StepBuffers& B, const DebugOut& dbg, cudaS
 // rows into its own region of Y, the y pass reads them back after a barrier;
 // the re-initialisation classifies into Y, scans rows (a thread per row) and
 // columns (a thread per column) in place and puts the signs back.  Same
-// arithmetic and FMA order as p_conv_xy; scans as scan_line_wrap without the
+// arithmetic and FMA order as p_conv_xy; scans without the
 // wrap.  The column passes are the shared ones.
 
 // Forward and backward min-plus scan of n magnitudes (stride st), in place.
-__device__ __forceinline__ void scan_line_serial(float* L, int n, int st) {
-    float f = L[0];
-    for (int j = 1; j < n; ++j) {
-        f = fminf(L[(long long)j * st], f + 1.0f);
-        L[(long long)j * st] = f;
-    }
-    for (int j = n - 2; j >= 0; --j) {
-        f = fminf(L[(long long)j * st], f + 1.0f);
-        L[(long long)j * st] = f;
-    }
-}
-
 template <int R, bool GRP>
 __global__ void __launch_bounds__(256)
 p_conv_xy_big(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
