@@ -127,16 +127,17 @@ struct StepState {                  // device-resident control block
     int n_slabs[kTiers];            // pass path: slab items (kSlab planes) per tier
     int slab_base[kTiers];
     long long step_limit;           // step groups: the member takes part while steps_done < step_limit
-    int bu_go;                      // the step's box update places offsets and items (set by its scan)
+    // the box update's sums while its CTAs add to them (zero between updates)
+    unsigned long long bu_elems, bu_done, bu_cells, bu_tier_cells[kTiers];
+    int bu_alive;
+    int bu_cls[kNumClasses];        // boxes per size class
+    int bu_items[3][kTiers];        // planes, column chunks, slabs per tier
+    unsigned bu_ticket;             // CTAs that have added theirs
     int pool_used;                  // neighbour-list pool entries taken by this step's lists
 };
 
-// The step's box update runs as three grid launches over chunks of
-// kBuChunk boxes: new boxes and per-chunk sums of kBuVals values, a scan of
-// the chunk sums (one CTA per context), then every box's arena offset and
-// work-item bases.
+// Boxes per CTA of the step's box update.
 constexpr int kBuChunk = 256;
-constexpr int kBuVals = 4 + kNumClasses + 4 * kTiers;
 
 __host__ __device__ inline int plane_stride(int nx, int ny) { return (nx * ny + 7) & ~7; }
 __host__ __device__ inline long long box_elems(const Box& b) {
@@ -209,7 +210,7 @@ struct StepBuffers {
     int2* plane_items;              // (box, local z), tier 0 then tier 1
     int2* chunk_items;              // (box, column chunk of kPassChunk columns)
     int2* slab_items;               // (box, first plane of a slab of kSlab planes)
-    int4* item_base;                // per box: first plane / chunk / slab item, tier (-1: no items)
+    int4* item_base;                // per box: first plane / chunk / slab item in its tier's lists, tier (-1: no items)
     long long plane_item_cap;       // entries (n_boxes * domain nz: a bound on sum nz)
     long long slab_item_cap;        // entries (n_boxes * ceil(domain nz / kSlab))
     long long chunk_item_cap;       // entries (n_boxes * 64 * 64 / kPassChunk)
@@ -219,7 +220,6 @@ struct StepBuffers {
     int pgrid[kTiers][5];           // persistent grid per tier and pass (conv_xy, conv_z ideal, conv_z physics, redist_xy, redist_z)
     int pocc[kTiers][5];            // resident CTAs per SM of those kernels (the grids' upper bound)
     int slab;                       // planes per slab item of p_redist_xy (kSlab unless autotuned)
-    long long* bu_part;             // box update: per chunk of kBuChunk boxes kBuVals sums, then their bases
     // field pass: boxes overlapping each domain tile of tile_x x (256 / tile_x) x kTileZ cells
     int tile_x;                     // 16, or 32 (set at creation; the lists are sized for it)
     int* tile_cnt;                  // [n_tiles]

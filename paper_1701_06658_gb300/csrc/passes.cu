@@ -2033,10 +2033,9 @@ cudaError_t launch_sweep_redist(const StepBuffers& B, const DebugOut& dbg, cudaS
 // rows into its own region of Y, the y pass reads them back after a barrier;
 // the re-initialisation classifies into Y, scans rows (a thread per row) and
 // columns (a thread per column) in place and puts the signs back.  Same
-// arithmetic and FMA order as p_conv_xy; scans without the
-// wrap.  The column passes are the shared ones.
+// arithmetic and FMA order as p_conv_xy; scans without the wrap.  The column
+// passes are the shared ones.
 
-// Forward and backward min-plus scan of n magnitudes (stride st), in place.
 template <int R, bool GRP>
 __global__ void __launch_bounds__(256)
 p_conv_xy_big(StepBuffers B1, GroupRef grp, Taps taps, int tier) {

@@ -224,3 +224,34 @@ def test_reinitialisation_of_the_step_s_own_phi_c(L, dims, G, bf16):
             box = O.Grain(g, tuple(int(v) for v in new[g, 3:0:-1]), np.zeros(tuple(int(v) for v in new[g, 6:3:-1])))
             kept = O.sample(was, O.box_positions(box, shape), shape, -7.0)[0]
             assert np.all(np.abs(phi[g] - kept) <= (2.0 ** -8 * np.abs(kept) if bf16 else 0.0)), g
+
+
+@pytest.mark.parametrize("dims,G", [((24, 26, 28), 1), ((40, 40, 40), 256), ((40, 44, 40), 257), ((64, 64, 70), 900)])
+def test_box_update_over_one_and_several_chunks(L, dims, G):
+    """The counts that the box update adds up over its chunks of boxes, against the boxes themselves (whole numbers:
+    equal), and the state of a context stepped alone (one launch closes the update) and in a group (two)."""
+    def make():
+        return L.Microstructure(*dims, G, seeds=I.voronoi_seeds(31, G, dims))
+
+    with make() as ms, make() as other:
+        done = 0
+        for _ in range(3):
+            b = ms.boxes().astype(np.int64)
+            done += int((b[:, 0] * b[:, 4] * b[:, 5] * b[:, 6]).sum())
+            ms.step(1, 1.0)
+            ms.sync()
+            b = ms.boxes().astype(np.int64)
+            cells = b[:, 0] * b[:, 4] * b[:, 5] * b[:, 6]
+            st = ms.stats()
+            assert st.cell_updates == done
+            assert st.alive == int(b[:, 0].sum()) and st.box_cells == int(cells.sum())
+            assert sum(st.pass_cells) == int(cells.sum())
+            side = np.maximum(b[:, 4], b[:, 5])
+            for t, (lo, hi) in enumerate(((0, 32), (32, 40), (40, 48), (48, 64), (64, 1 << 30))):
+                assert st.pass_cells[t] == int(cells[(side > lo) & (side <= hi)].sum())
+        with L.Group([other]) as g:
+            g.step(3, 1.0)
+        other.sync()
+        assert other.stats().cell_updates == done
+        assert np.array_equal(ms.boxes(), other.boxes())
+        assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(other.ctx))
