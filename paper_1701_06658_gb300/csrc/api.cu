@@ -720,6 +720,13 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         }
         if ((r = dalloc(c, &c->B.scratch, (size_t)std::max(total, 32LL))) != LSGG_OK) return bail(r);
     }
+    if (c->B.use_passes) {
+        // slab items enough to go round: a shorter slab loads and classifies
+        // more planes twice, a longer one leaves SMs idle
+        long long planes = 0;
+        for (const Box& b : hb) planes += b.nz;
+        while (c->B.slab > kMinSlab && planes < (long long)kSlabItemsPerSm * c->B.n_sm * c->B.slab) c->B.slab /= 2;
+    }
     if ((r = relayout(c)) != LSGG_OK) return bail(r);
     c->phys.kind = cfg_in->physics;
     c->phys.energy = c->d_energy;
@@ -1072,14 +1079,14 @@ static int apply_pass_tuning(lsgg_ctx* c, const int (&ctas)[kTiers][5], int slab
 
 // Autotuner of the pass path: trials of steps_per_trial profiled steps each
 // with (a) every grid at its resident maximum and the default slab, (b) every
-// grid at half of it, (c, d) slabs of 4 and 16 planes; per tier and pass the
-// faster grid of (a, b), and the slab with the least re-initialisation
-// plane-pass time over the tiers.  All settings give bit-identical steps.
+// grid at half of it, (c, d) slabs of half and twice the default; per tier and
+// pass the faster grid of (a, b), and the slab with the least
+// re-initialisation plane-pass time over the tiers.  All settings give bit-identical steps.
 static int autotune_passes(lsgg_ctx* c, int32_t steps_per_trial, double dt) {
     int full[kTiers][5], half[kTiers][5];
     for (int t = 0; t < kTiers; ++t)
         for (int k = 0; k < 5; ++k) { full[t][k] = c->B.pocc[t][k]; half[t][k] = std::max(1, c->B.pocc[t][k] / 2); }
-    const int slabs[4] = {kSlab, kSlab, kMinSlab, 2 * kSlab};
+    const int slabs[4] = {kSlab, kSlab, kSlab / 2, 2 * kSlab};
     double ms[4][kTiers * 4 + 2] = {};
     c->profiling = true;
     for (int trial = 0; trial < 4; ++trial) {

@@ -37,7 +37,14 @@ constexpr int kTiers = 5;               // pass path: boxes with x, y sides <= 3
 constexpr int kFewBoxes = 2048;         // up to this many boxes, kernels of a CTA per box take a cluster per box
 constexpr int kPassChunk = 256;         // columns per column item of the pass path
 constexpr int kSlab = 8;                // planes per slab item of the pass path (default; autotuned)
-constexpr int kMinSlab = 4;             // the smallest slab the autotuner tries (sizes the slab item list)
+constexpr int kMinSlab = 2;             // the smallest slab (sizes the slab item list)
+// The slab is halved while the initial boxes give fewer slab items per SM than
+// this.  Measured on GB300, a step with the slab so found and with 8 planes:
+// 32^3 / 20 grains 0.093 and 0.112 ms, 64^3 / 50 0.089 and 0.108.  With the
+// line at 8 or 16 149 x 97 x 61 / 263 would gain too (0.164 against 0.175 ms),
+// but a served mix of 24 requests, whose groups fill the GPU, takes 164 or
+// 176 ms (at 4 158, with 8 planes 160).
+constexpr int kSlabItemsPerSm = 4;
 constexpr int kTileThreads = 256;       // columns of a field-pass tile, one per thread
 constexpr int kTileZ = 8;               // planes of a field-pass tile (its columns: StepBuffers::tile_x)
 constexpr long long kWideTileCells = 96LL << 20;   // domains above this with physics: 32-column tiles
@@ -219,7 +226,7 @@ struct StepBuffers {
     int tier_threads[kTiers];       // threads per CTA of the plane passes (= tier side)
     int pgrid[kTiers][5];           // persistent grid per tier and pass (conv_xy, conv_z ideal, conv_z physics, redist_xy, redist_z)
     int pocc[kTiers][5];            // resident CTAs per SM of those kernels (the grids' upper bound)
-    int slab;                       // planes per slab item of p_redist_xy (kSlab unless autotuned)
+    int slab;                       // planes per slab item of the plane passes
     // field pass: boxes overlapping each domain tile of tile_x x (256 / tile_x) x kTileZ cells
     int tile_x;                     // 16, or 32 (set at creation; the lists are sized for it)
     int* tile_cnt;                  // [n_tiles]

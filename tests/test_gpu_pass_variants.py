@@ -255,3 +255,24 @@ def test_box_update_over_one_and_several_chunks(L, dims, G):
         assert other.stats().cell_updates == done
         assert np.array_equal(ms.boxes(), other.boxes())
         assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(other.ctx))
+
+
+@pytest.mark.parametrize("dims,G", [((24, 24, 24), 4), ((64, 60, 64), 110), ((96, 90, 100), 300)])
+def test_slab_depth_follows_the_box_planes(L, dims, G):
+    """The depth that the context starts with, and the same bits as with the depths that a tuning tries."""
+    import torch
+    seeds = I.voronoi_seeds(37, G, dims)
+    with L.Microstructure(*dims, G, seeds=seeds) as ms, L.Microstructure(*dims, G, seeds=seeds) as tuned:
+        slab = 8
+        planes = int(ms.boxes()[:, 6].sum())
+        while slab > 2 and planes < 4 * torch.cuda.get_device_properties(0).multi_processor_count * slab:
+            slab //= 2
+        assert L.pass_tuning(ms.ctx)["slab"] == slab
+        ms.step(6, 1.0)
+        ms.sync()
+        L.autotune(tuned.ctx, 1, 1.0)                    # four steps
+        assert L.pass_tuning(tuned.ctx)["slab"] in (4, 8, 16)
+        tuned.step(2, 1.0)
+        tuned.sync()
+        assert np.array_equal(ms.boxes(), tuned.boxes())
+        assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(tuned.ctx))
