@@ -1,0 +1,66 @@
+"""The device memory of contexts that come and go: given back but for a bounded rest, sound for contexts of several
+threads at once, each on its own stream."""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_1701_06658_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_1701_06658_gb300 import lsgg
+    lsgg.lib()
+    return lsgg
+
+
+def _run(L, seed):
+    n = 24 + 8 * (seed % 4)
+    with L.Microstructure(n, n + 2, n + 4, 12, seeds=I.voronoi_seeds(seed, 12, (n, n + 2, n + 4))) as ms:
+        ms.step(4, 1.0)
+        ms.sync()
+        return ms.boxes(), L.get_phi(ms.ctx), ms.grain_volumes()
+
+
+def test_threads_reuse_each_other_s_memory(L):
+    want = {s: _run(L, s) for s in range(8)}
+    got, errors = {}, []
+
+    def work(first):
+        try:
+            for k in range(3):
+                for s in range(8):
+                    got[first, k, s] = _run(L, (s + first) % 8)
+        except Exception as e:                       # seen by the asserting thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    for (first, _, s), r in got.items():
+        for a, b in zip(r, want[(s + first) % 8]):
+            assert np.array_equal(a, b)
+
+
+def test_memory_is_given_back(L):
+    import torch
+    _run(L, 1)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    n, G = 128, 600
+    mss = [L.Microstructure(n, n, n, G, seeds=I.voronoi_seeds(k, G, (n, n, n))) for k in range(6)]
+    held = sum(ms.stats().device_bytes for ms in mss)
+    for ms in mss:
+        ms.close()
+    torch.cuda.synchronize()
+    assert held > 2 << 30                            # more than the pool keeps without contexts
+    assert torch.cuda.mem_get_info()[0] >= free - (1 << 30) - (64 << 20)
