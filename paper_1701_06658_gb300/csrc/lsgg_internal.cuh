@@ -19,7 +19,7 @@
 //   classes    per size class a work list of box indices and a queue counter
 //              per kernel; persistent CTAs pull boxes from the queue.
 //   items      pass path: per tier a list of (box, plane), of (box, slab of
-//              kSlab planes) and of (box, column chunk) work items, rebuilt by
+//              planes) and of (box, column chunk) work items, rebuilt by
 //              every box update.
 #pragma once
 
@@ -131,7 +131,7 @@ struct StepState {                  // device-resident control block
     int plane_base[kTiers];
     int chunk_base[kTiers];
     long long tier_cells[kTiers];   // box cells per tier in `cur`
-    int n_slabs[kTiers];            // pass path: slab items (kSlab planes) per tier
+    int n_slabs[kTiers];            // pass path: slab items per tier
     int slab_base[kTiers];
     long long step_limit;           // step groups: the member takes part while steps_done < step_limit
     // the box update's sums while its CTAs add to them (zero between updates)
@@ -216,10 +216,10 @@ struct StepBuffers {
     float* Z;
     int2* plane_items;              // (box, local z), tier 0 then tier 1
     int2* chunk_items;              // (box, column chunk of kPassChunk columns)
-    int2* slab_items;               // (box, first plane of a slab of kSlab planes)
+    int2* slab_items;               // (box, first plane of the slab)
     int4* item_base;                // per box: first plane / chunk / slab item in its tier's lists, tier (-1: no items)
     long long plane_item_cap;       // entries (n_boxes * domain nz: a bound on sum nz)
-    long long slab_item_cap;        // entries (n_boxes * ceil(domain nz / kSlab))
+    long long slab_item_cap;        // entries (n_boxes * ceil(domain nz / kMinSlab))
     long long chunk_item_cap;       // entries (n_boxes * 64 * 64 / kPassChunk)
     int use_passes;
     int tier_side[kTiers];

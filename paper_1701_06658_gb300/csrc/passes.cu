@@ -8,12 +8,13 @@
 // serialised a whole box along z.  The fields between passes go through HBM:
 //   k_bin       per box: list it in every domain tile it overlaps; reset its
 //               positive bounding box
-//   p_conv_xy   (box, plane): bulk copy of the plane of phi in the old layout,
-//               staged into the new layout (-eps outside), x and y passes in
-//               shared memory                                     -> Z = xy-convolved
-//   p_conv_z    (box, columns): z pass from the column in registers, velocity
-//               correction (Read-Shockley pairs from a per-box hash of the
-//               step's neighbour list), clamp                     -> Y = phi_p
+//   p_conv_xy   (box, slab): bulk copies of its planes of phi in the old layout,
+//               staged in pairs into the new layout (-eps outside), x and y
+//               passes in shared memory, two planes an FMA        -> Z = xy-convolved
+//   p_conv_z    (box, columns): z pass from the column in registers (physics:
+//               as running sums over batches of planes), velocity correction
+//               (Read-Shockley pairs from a per-box hash of the step's
+//               neighbour list), clamp                            -> Y = phi_p
 //   p_field     (domain tile): the two largest (phi_p, grain) per cell over
 //               the tile's boxes in registers (stored in T as (phi_p, -id)
 //               keys only on request, B.keep_field); then
@@ -21,8 +22,8 @@
 //               the tile                                          -> Z = phi_c
 //   p_redist_xy (box, slab): plane ring filled by bulk copies; reference cells
 //               with their planar-exact distances, y and x taxicab scans -> Y
-//   p_redist_z  (box, columns): the column in registers, z taxicab scans,
-//               signs, positive bounding box                      -> X = phi
+//   p_redist_z  (box, columns): the column in registers (a variant per eight
+//               planes), z taxicab scans, signs, positive bounding box -> X = phi
 // The field pass replaces the box-streaming kernels' atomic scatter: each
 // domain cell's top-2 is built by the one thread that owns the cell, so the
 // step has no atomics on the field.  The work-item lists are written by the
@@ -1257,7 +1258,7 @@ __device__ __forceinline__ void scan_seg_wrap(float* line, int st, int n, int x0
 }
 
 // Plane pass of the re-initialisation: a CTA of NT = 4 * SIDE threads takes
-// one (box, slab of kSlab planes) item at a time and walks its planes in z
+// one (box, slab of planes) item at a time and walks its planes in z
 // order.  Planes of phi_c stream into a 3-slot shared-memory ring by bulk
 // copies (a box plane is contiguous and 16-byte aligned), plane z + 2 being
 // fetched while plane z is processed.  Thread (r, s) owns cells [s L, s L +

@@ -12,8 +12,9 @@
 //               sign-blocked min-plus transform, x and y in the plane, z as a
 //               forward sweep plus a 6-plane backward window; clamp; positive
 //               bounding box of the box.
-//   k_box_update  Secs. 2.1.3 / 3.1: new box = bbox{phi > 0} + halo, arena
-//               offsets by a block-wide scan, size classes and work queues.
+//   k_bu        Secs. 2.1.3 / 3.1: new box = bbox{phi > 0} + halo, arena
+//               offsets, size classes, work queues and items (k_box_update:
+//               the layout alone, by one CTA).
 //
 // One CTA owns one box at a time and streams it plane by plane; CTAs of a
 // size class pull boxes from a device queue (persistent grid).  Outside its
