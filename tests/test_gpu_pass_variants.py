@@ -276,3 +276,25 @@ def test_slab_depth_follows_the_box_planes(L, dims, G):
         tuned.sync()
         assert np.array_equal(ms.boxes(), tuned.boxes())
         assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(tuned.ctx))
+
+
+@pytest.mark.parametrize("side", [32, 33, 40, 41, 48, 49, 64, 65])
+def test_steps_leave_out_only_tiers_without_boxes(L, side):
+    """Replayed steps launch the tiers that the domain's boxes can be in; profiled steps launch every tier.  The same
+    bits for boxes that span the domain's longer side, alone and in a group with a smaller domain."""
+    dims, G = (side, 24, 20), 2
+    seeds = np.array([[0.0, 6.0, 3.0], [0.0, 18.0, 13.0]])       # both grains span x
+    small = I.voronoi_seeds(42, 4, (24, 24, 24))
+    with L.Microstructure(*dims, G, seeds=seeds) as ms, L.Microstructure(*dims, G, seeds=seeds) as every, \
+            L.Microstructure(*dims, G, seeds=seeds) as member, L.Microstructure(24, 24, 24, 4, seeds=small) as other:
+        L.profile(every.ctx, True)
+        ms.step(4, 1.0)
+        every.step(4, 1.0)
+        with L.Group([other, member]) as g:
+            g.step(4, 1.0)
+        for m in (ms, every, member):
+            m.sync()
+        assert int(every.boxes()[:, 4].max()) == side
+        for m in (ms, member):
+            assert np.array_equal(m.boxes(), every.boxes())
+            assert np.array_equal(L.get_phi(m.ctx), L.get_phi(every.ctx))
