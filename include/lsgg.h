@@ -357,8 +357,8 @@ int lsgg_autotune(lsgg_ctx* ctx, int32_t steps_per_trial, double dt, int32_t* ch
 /* The pass path's current tuning: ctas_per_sm (optional, 4 * LSGG_PASS_TIERS
  * int32) the CTAs per SM of the persistent grids of p_conv_xy, p_conv_z,
  * p_redist_xy and p_redist_z of each tier, slab (optional) the planes per slab
- * item of the plane passes (before a tuning 8, or 4 or 2 for microstructures
- * of few box planes); -1 off the pass path. */
+ * item of the plane passes (before a tuning 16, 8, 4 or 2 by the number of
+ * box planes); -1 off the pass path. */
 int lsgg_pass_tuning(lsgg_ctx* ctx, int32_t* ctas_per_sm, int32_t* slab);
 int lsgg_kernel_times(lsgg_ctx* ctx, double* out_ms, int64_t* out_count);
 

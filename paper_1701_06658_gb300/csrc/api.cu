@@ -839,6 +839,7 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         // more planes twice, a longer one leaves SMs idle
         long long planes = 0;
         for (const Box& b : hb) planes += b.nz;
+        if (planes >= (long long)kDeepItemsPerSm * c->B.n_sm * kDeepSlab) c->B.slab = kDeepSlab;
         while (c->B.slab > kMinSlab && planes < (long long)kSlabItemsPerSm * c->B.n_sm * c->B.slab) c->B.slab /= 2;
     }
     if ((r = relayout(c)) != LSGG_OK) return bail(r);

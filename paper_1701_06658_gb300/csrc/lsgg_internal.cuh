@@ -45,6 +45,12 @@ constexpr int kMinSlab = 2;             // the smallest slab (sizes the slab ite
 // but a served mix of 24 requests, whose groups fill the GPU, takes 164 or
 // 176 ms (at 4 158, with 8 planes 160).
 constexpr int kSlabItemsPerSm = 4;
+// Slabs of 16 where they still give this many items per SM: fewer planes are
+// loaded and classified twice.  A step on GB300 with 8 and with 16 planes: 256^3 /
+// 5000 grains 1.780 and 1.760 ms, 384^3 magnetic 7.48 and 7.39, 512^3
+// Read-Shockley 20.50 and 20.38; 32 items per SM leave 191^3 / 2077 (0.769
+// against 0.760) out.
+constexpr int kDeepSlab = 16, kDeepItemsPerSm = 16;
 constexpr int kTileThreads = 256;       // columns of a field-pass tile, one per thread
 constexpr int kTileZ = 8;               // planes of a field-pass tile (its columns: StepBuffers::tile_x)
 constexpr long long kWideTileCells = 96LL << 20;   // domains above this with physics: 32-column tiles

@@ -298,3 +298,19 @@ def test_steps_leave_out_only_tiers_without_boxes(L, side):
         for m in (ms, member):
             assert np.array_equal(m.boxes(), every.boxes())
             assert np.array_equal(L.get_phi(m.ctx), L.get_phi(every.ctx))
+
+
+@pytest.mark.parametrize("dims,G", [((128, 126, 140), 2600)])
+def test_deep_slabs_for_many_planes(L, dims, G):
+    import torch
+    seeds = I.voronoi_seeds(43, G, dims)
+    with L.Microstructure(*dims, G, seeds=seeds) as ms, L.Microstructure(*dims, G, seeds=seeds) as tuned:
+        n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+        assert (L.pass_tuning(ms.ctx)["slab"] == 16) == (int(ms.boxes()[:, 6].sum()) >= 16 * 16 * n_sm)
+        ms.step(5, 1.0)
+        ms.sync()
+        L.autotune(tuned.ctx, 1, 1.0)                # four steps with 8, 8, 4 and 16 planes
+        tuned.step(1, 1.0)
+        tuned.sync()
+        assert np.array_equal(ms.boxes(), tuned.boxes())
+        assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(tuned.ctx))
