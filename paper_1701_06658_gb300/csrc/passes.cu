@@ -323,7 +323,10 @@ p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
                 if (t == 0) {
                     atomicExch(&B.st->status, LSGG_ERR_TIMEOUT);
                     atomicExch(&B.st->halt, 1);
-                    mbar_wait(bar, phase);
+                    // the copies of this phase, unless this thread saw them
+                    // complete (its phase is the next one then, which no copy
+                    // was issued for)
+                    if (!ok) mbar_wait(bar, phase);
                 }
                 __syncthreads();
                 return;

@@ -107,3 +107,29 @@ def test_step_waits_give_up_and_the_context_recovers(L):
         assert b.stats().steps_done == 3
         assert np.array_equal(b.boxes(), want_boxes)
         assert np.array_equal(L.get_phi(b.ctx), want_phi)
+
+
+@pytest.mark.parametrize("limit", [1, 2, 8])
+def test_waits_that_some_threads_complete(L, limit):
+    """A poll limit that some threads of a CTA reach and others do not: a pass that gives up drains only what is
+    still in flight, so the step ends at once (a drain of a phase without copies would poll four million times);
+    after it, with the default limit, the state is that of a context that never gave up."""
+    import time
+    from paper_1701_06658_gb300 import inputs as I
+    N, G = 32, 20                                    # boxes of one tier: no other tier's passes run on meanwhile
+    seeds = I.voronoi_seeds(1, G, (N, N, N))
+    with L.Microstructure(N, N, N, G, seeds=seeds) as a, L.Microstructure(N, N, N, G, seeds=seeds) as b:
+        b.sync()
+        L.debug_set_wait_limit(b.ctx, limit)
+        t0 = time.monotonic()
+        for _ in range(10):
+            b.step(1, 1.0)
+            assert L.lib().lsgg_sync(b.ctx, -1) in (L.OK, L.ERR_TIMEOUT)
+        assert time.monotonic() - t0 < 1.0           # ten steps of about 0.1 ms
+        L.debug_set_wait_limit(b.ctx, -1)
+        b.step(2, 1.0)
+        b.sync()
+        a.step(b.stats().steps_done, 1.0)
+        a.sync()
+        assert np.array_equal(a.boxes(), b.boxes())
+        assert np.array_equal(L.get_phi(a.ctx), L.get_phi(b.ctx))
