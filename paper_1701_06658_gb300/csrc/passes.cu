@@ -262,6 +262,7 @@ p_conv_xy(StepBuffers B1, GroupRef grp, Taps taps, int tier) {
         const StepBuffers& Bx = member<GRP>(B1, grp, s_gb, i, l);
         const int2 itx = list_item<GRP>(Bx, items, kItemSlabs, tier, i, l);
         const Box nb = Bx.cur[itx.x], ob = Bx.prev[itx.x];
+        if (max(ob.nx, ob.ny) > SIDE) return;           // its planes overrun the slots: refused below, nothing in flight
         fetch(Bx, ob, wrap_near(nb.oz - ob.oz, Bx.dom.nz), itx.y, min(itx.y + Bx.slab, nb.nz));
     };
     if (blockIdx.x < n_items) fetch_item(blockIdx.x);
