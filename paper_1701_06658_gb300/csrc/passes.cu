@@ -959,7 +959,10 @@ p_field(StepBuffers B1, GroupRef grp, PhysicsDev phys, DebugOut dbg) {
     __shared__ int s_gb[GRP ? kMaxGroup + 1 : 1];
     extern __shared__ float s_val[];                // SLOTS x kTileZ x kTileThreads
     if (!GRP && halted(B1)) return;
-    if (IDS && threadIdx.x >= kTileCap && threadIdx.x < 256) s_id[threadIdx.x] = -1;
+    if (IDS) {                                      // before the first tile's reads: one without boxes has no barrier
+        if (threadIdx.x >= kTileCap && threadIdx.x < 256) s_id[threadIdx.x] = -1;
+        __syncthreads();
+    }
     const int n_all = GRP ? group_scan(grp, kItemTiles, 0, true, s_gb) : B1.n_tiles;
     const int lx = threadIdx.x % TX, ly = threadIdx.x / TX;
     for (int gtile = blockIdx.x; gtile < n_all; gtile += gridDim.x) {

@@ -314,3 +314,32 @@ def test_deep_slabs_for_many_planes(L, dims, G):
         tuned.sync()
         assert np.array_equal(ms.boxes(), tuned.boxes())
         assert np.array_equal(L.get_phi(ms.ctx), L.get_phi(tuned.ctx))
+
+
+@pytest.mark.parametrize("kind", ["ideal", "magnetic"])
+def test_field_pass_over_tiles_without_boxes(L, kind):
+    """A state that covers one corner of the domain: the other tiles list no box, many CTAs' first tile among them.
+    The grains around the boxes' cells are the oracle's, those of the empty tiles none."""
+    from oracle import lsgg_oracle as O
+    n = 96
+    dims = (n, n, n)
+    kw = {"physics": L.PHYSICS_MAGNETIC, "energy": np.zeros(2)} if kind == "magnetic" else {}
+    boxes = np.zeros((2, 7), np.int32)
+    boxes[0] = (1, 4, 4, 4, 22, 20, 24)
+    boxes[1] = (1, 12, 4, 4, 22, 20, 24)
+    z, y, x = np.meshgrid(np.arange(24), np.arange(20), np.arange(22), indexing="ij")
+    ball = np.clip(6.0 - np.sqrt((x - 11.0) ** 2 + (y - 10.0) ** 2 + (z - 12.0) ** 2), -7.0, 7.0).astype(np.float32)
+    phi = {0: ball, 1: ball.copy()}
+    idf = {g: np.full(ball.shape, 1 - g, np.int32) for g in phi}
+    with L.Microstructure(*dims, 2, seeds=np.array([[15.0, 14.0, 16.0], [23.0, 14.0, 16.0]]), **kw) as ms:
+        ms.set_state(boxes, phi, idf)
+        L.keep_field(ms.ctx, True)
+        was, (phip, m, idm, phic, _) = ms.debug_step(1.0)
+        near = L.grain_neighbours(ms.ctx, 2)
+    grains = [O.Grain(g, (4, 4, int(was[g, 1])), phip[g].astype(np.float64)) for g in (0, 1)]
+    pp = {g: phip[g].astype(np.float64) for g in (0, 1)}
+    for g in (0, 1):
+        rm, rid = O.neighbour_max(g, grains, pp, dims, 7.0)
+        assert np.array_equal(m[g], rm.astype(np.float32)) and np.array_equal(idm[g], rid)
+        assert np.array_equal(phic[g], np.float32(0.5) * (phip[g] - m[g]))
+        assert list(near[g]) == [1 - g]
