@@ -731,7 +731,10 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
     long long bin_bytes = 0;
     float4* d_bpts = nullptr;
     int *d_bids = nullptr, *d_bstart = nullptr;
-    int2* d_sdf_items = nullptr;                 // work items of the initial functions
+    // work items of the initial functions; the host's stay until the stream has
+    // been waited for (a copy from pageable memory may return before it is done)
+    int2* d_sdf_items = nullptr;
+    std::vector<int2> sdf_items;
     long long sdf_bytes = 0;
     unsigned* d_occ = nullptr;                   // label field: per grain and axis the positions it holds
     const int occ_words = (std::max(D.nx, std::max(D.ny, D.nz)) + 31) / 32;
@@ -880,17 +883,16 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         long long all = 0;
         for (const Box& b : hb) all += b.nx > 0 ? (long long)((b.nx + 3) / 4) * b.ny * b.nz : 0;
         const int groups = (int)std::min(4096LL, std::max(256LL, all / (8LL * c->B.n_sm) / 256 * 256));
-        std::vector<int2> items;
         for (int b = 0; b < G; ++b) {
             if (hb[b].nx <= 0) continue;
             const int n = (hb[b].nx + 3) / 4 * hb[b].ny * hb[b].nz;
-            for (long long q = 0; q < n; q += groups) items.push_back(make_int2(b, (int)q));
+            for (long long q = 0; q < n; q += groups) sdf_items.push_back(make_int2(b, (int)q));
         }
-        if ((r = dalloc(c, &d_sdf_items, items.size())) != LSGG_OK) return bail(r);
-        sdf_bytes = (long long)std::max<size_t>(items.size() * sizeof(int2), 16);
-        if (cudaMemcpyAsync(d_sdf_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, c->stream) !=
+        if ((r = dalloc(c, &d_sdf_items, sdf_items.size())) != LSGG_OK) return bail(r);
+        sdf_bytes = (long long)std::max<size_t>(sdf_items.size() * sizeof(int2), 16);
+        if (cudaMemcpyAsync(d_sdf_items, sdf_items.data(), sdf_items.size() * sizeof(int2), cudaMemcpyHostToDevice, c->stream) !=
                 cudaSuccess ||
-            launch_sdf(D, d_sdf_items, (int)items.size(), groups, c->B.cur, c->d_seeds, c->d_weights, d_bits, wpr,
+            launch_sdf(D, d_sdf_items, (int)sdf_items.size(), groups, c->B.cur, c->d_seeds, c->d_weights, d_bits, wpr,
                        c->B.bf16 ? c->B.Y : c->B.X, c->B.IDF, &c->B.st->status, c->stream) != cudaSuccess)
             return bail(CUDA_FAIL());
         if (c->B.bf16 && launch_f32_to_state(c->B.Y, c->B.X, c->B.cap, c->stream) != cudaSuccess)
