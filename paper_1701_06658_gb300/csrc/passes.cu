@@ -482,9 +482,12 @@ __device__ __noinline__ void rs_pair_out_of_line(const PhysicsDev& phys, int i, 
 // energies -- all in flight together, at four CTAs per SM instead of two.
 // Cells without a pair take the convolution c, others phi + w (c - phi) + M
 // (e_j - e_i) dt: Read-Shockley (RS) with w from the box's pair hash and no
-// bulk term, magnetic with w = M = 1.
+// bulk term, magnetic with w = M = 1.  False: an id of the column was not in
+// the hash, whose list should hold every id of the box's ID-field; the column is
+// then the general form's, which evaluates such a pair (a call in the loop here
+// would spill a quarter of its registers).
 template <int R, bool RS>
-__device__ __forceinline__ void conv_fir_phys(const StepBuffers& B, const PhysicsDev& phys, const float* zc, float* yc,
+__device__ __forceinline__ bool conv_fir_phys(const StepBuffers& B, const PhysicsDev& phys, const float* zc, float* yc,
                                               int nz, int ps, const float (&g)[2 * R + 1], float cconst, float eps,
                                               long long o_old, int ps_old, int ozl0, int onz, int dnz, bool in_old, float ei,
                                               const int2* hash) {
@@ -503,6 +506,7 @@ __device__ __forceinline__ void conv_fir_phys(const StepBuffers& B, const Physic
     const float* const xo = B.X + (bf16 ? 0 : o_old);
     const __nv_bfloat16* const xb = reinterpret_cast<const __nv_bfloat16*>(B.X) + o_old;
     const int* const jo = B.IDF + o_old;
+    int found = 0;                                         // negative once a search ended on an empty slot
     for (int base = 0; base < nz + R; base += kZB) {
         float v[kZB], p0[kZB], ej[RS ? 1 : kZB];
         int jj[kZB];
@@ -534,14 +538,15 @@ __device__ __forceinline__ void conv_fir_phys(const StepBuffers& B, const Physic
             const int j = jj[u];
             if (j >= 0) {
                 if constexpr (RS) {
-                    // the list holds every id of the box's ID-field; at most
-                    // half full, so an empty slot would end the search
+                    // at most half full, so an empty slot ends the search of a
+                    // missing id
                     unsigned h = zhash(j);
                     int2 e = hash[h];
                     while (e.x != j && e.x >= 0) {
                         h = (h + 1) & (kZHash - 1);
                         e = hash[h];
                     }
+                    found |= e.x;
                     val = fmaf(__int_as_float(e.y), val - p0[u], p0[u]);
                 } else {
                     val = fmaf(ej[u] - ei, phys.dt, p0[u] + (val - p0[u]));
@@ -550,6 +555,7 @@ __device__ __forceinline__ void conv_fir_phys(const StepBuffers& B, const Physic
             yc[(size_t)((unsigned)zo * (unsigned)ps)] = fminf(fmaxf(val, -eps), eps);
         }
     }
+    return found >= 0;
 }
 
 // The z pass of one column in its general form (periodic or long columns; with
@@ -742,9 +748,9 @@ p_conv_z(const __grid_constant__ StepBuffers B1, GroupRef grp, const __grid_cons
                 const bool in_old = oxl < ob.nx && oyl < ob.ny;
                 const long long o_old = ob.off + (in_old ? (long long)oyl * ob.nx + oxl : 0);
                 const int ozl0 = wrap_near(nb.oz - ob.oz, dnz);
-                conv_fir_phys<R, rs>(B, phys, zc, yc, nz, ps, g, cconst1, eps, o_old, ps_old, ozl0, ob.nz, dnz, in_old,
-                                     rs ? 0.0f : phys.energy[b], s_h);
-                continue;
+                if (conv_fir_phys<R, rs>(B, phys, zc, yc, nz, ps, g, cconst1, eps, o_old, ps_old, ozl0, ob.nz, dnz, in_old,
+                                         rs ? 0.0f : phys.energy[b], s_h))
+                    continue;
             }
         }
         conv_z_general<R, PHYS>(B, phys, taps, tab, s_h, hash_n, b, c);

@@ -343,3 +343,29 @@ def test_field_pass_over_tiles_without_boxes(L, kind):
         assert np.array_equal(m[g], rm.astype(np.float32)) and np.array_equal(idm[g], rid)
         assert np.array_equal(phic[g], np.float32(0.5) * (phip[g] - m[g]))
         assert list(near[g]) == [1 - g]
+
+
+def test_neighbour_collection_of_many_boxes(L):
+    """More boxes than take eight CTAs each: phi_p of the second step, whose pairs' weights come from the lists that
+    two CTAs a box collect from the first step's ID-field, within the parity tests' 3e-5."""
+    from oracle import lsgg_oracle as O
+    from tests.parity import oracle_from_gpu
+    dims, G = (72, 68, 70), 2100
+    quats = I.random_quaternions(14, G)
+    ph = O.read_shockley_physics(quats)
+    shape = (dims[2], dims[1], dims[0])
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(14, G, dims), quats=quats,
+                          physics=L.PHYSICS_READ_SHOCKLEY) as ms:
+        old, (_, _, idm, _, _) = ms.debug_step(1.0)
+        boxes, phi = ms.boxes(), ms.phi()
+        _, (phip, *_rest) = ms.debug_step(1.0)
+    ref = oracle_from_gpu(shape, boxes, phi, None, ph)
+    taps = O.heat_kernel_taps(1.0, 5)
+    seen = 0
+    for g in list(phip)[::9]:
+        was = O.Grain(g, (int(old[g, 3]), int(old[g, 2]), int(old[g, 1])), idm[g].astype(np.float64))
+        ref.grains[g].idf = O.sample(was, O.box_positions(ref.grains[g], shape), shape, -1)[0].astype(np.int64)
+        seen = max(seen, len(np.unique(ref.grains[g].idf)))
+        want = O.predict(ref.grains[g], shape, taps, 7.0, ph, 1.0)
+        assert np.max(np.abs(phip[g] - want)) <= 3e-5, g
+    assert seen > 16                                 # lists of some length
