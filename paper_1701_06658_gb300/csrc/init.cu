@@ -544,7 +544,8 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
     // the box's cells as consecutive integers q = shift + l whose displacement
     // q - s_i stays within half a period (fast), its first and last values
     int shift[3];
-    float first[3], last[3], asum = 0.0f;
+    double first[3], last[3];
+    float asum = 0.0f, ssum = 0.0f;
     bool fast = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -552,18 +553,19 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
         const double d0 = (double)o[a] - si[a];
         if (d0 > 0.5 * Nd[a]) shift[a] -= Ni[a];
         else if (d0 < -0.5 * Nd[a]) shift[a] += Ni[a];
-        first[a] = (float)((double)shift[a] - si[a]);
-        last[a] = first[a] + (float)(bn[a] - 1);
-        fast = fast && first[a] > -0.5f * Nf[a] + 2e-2f && last[a] < 0.5f * Nf[a] - 2e-2f && Ni[a] < (1 << 22);
-        asum += fmaxf(fabsf(first[a]), fabsf(last[a]));
+        first[a] = (double)shift[a] - si[a];
+        last[a] = first[a] + (double)(bn[a] - 1);
+        fast = fast && first[a] > -0.5 * Nd[a] + 2e-2 && last[a] < 0.5 * Nd[a] - 2e-2 && Ni[a] < (1 << 22);
+        asum += (float)fmax(fabs(first[a]), fabs(last[a]));
+        ssum += fabsf((float)si[a]);
     }
     for (int k = t; k < cnt; k += kSdfThreads) {
         const int j = s_nb[k];
         const double wj = weights ? weights[j] : 0.0;
         const double d0 = min_image(si[0] - seeds[3 * j], Nd[0]), d1 = min_image(si[1] - seeds[3 * j + 1], Nd[1]),
                      d2 = min_image(si[2] - seeds[3 * j + 2], Nd[2]);
-        const float df[3] = {(float)d0, (float)d1, (float)d2};
-        s_d[k] = make_float4(df[0], df[1], df[2], (float)(wj - wi));
+        const double dd[3] = {d0, d1, d2};
+        s_d[k] = make_float4((float)d0, (float)d1, (float)d2, (float)(wj - wi));
         const double len = sqrt(fma(d0, d0, fma(d1, d1, d2 * d2)));
         SdfPair q;
         q.n0 = d0 / len;
@@ -578,7 +580,7 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
         // one image of the neighbour's seed for every cell of the box
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            fast = fast && fabsf(first[a] + df[a]) < 0.5f * Nf[a] - 2e-2f && fabsf(last[a] + df[a]) < 0.5f * Nf[a] - 2e-2f;
+            fast = fast && fabs(first[a] + dd[a]) < 0.5 * Nd[a] - 2e-2 && fabs(last[a] + dd[a]) < 0.5 * Nd[a] - 2e-2;
         fast = fast && fabsf(f.w) < 1e6f;
         atomicMax(reinterpret_cast<int*>(&s_cmax), __float_as_int(fabsf(f.w)));
     }
@@ -691,10 +693,19 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
         return (float)(best == DBL_MAX ? eps : (best < -eps ? -eps : (best > eps ? eps : best)));
     };
 
-    // FP32 screening error: n and a rounded, three FMAs; double-float error:
-    // s_i to 48 bits, the products' and sums' last places, and the FP64 form's own
+    // Error bounds, with A = asum >= |n . a|, S = ssum = the sum of |s_i|, C =
+    // s_cmax >= |c| and u = 2^-24 (half an FP32 ulp, relative).
+    // Screening: n, a and c rounded (u (2 A + C)), three FMAs (3 u (A + C)); E
+    // is twice that.  a is the displacement from the FP64 seed, rounded once:
+    // from the seed rounded to FP32, as u S alone exceeds E in wide domains.
+    // Double-float, in u^2: s_i beyond 48 bits and its low part's difference
+    // (A + 2 S), n and c beyond 48 bits (A + C), the product of the low parts
+    // (A), the products' rests (each u |n a|) added up (2 A), six FMAs on at most
+    // 3 u A (18 A), the sums' rests added up (5 A + C), c's low part added (3 A
+    // + 2 C) and the total (6 A + 2 C), the test's own rest + edd (A + C), and
+    // the FP64 form's roundings (below A / 4 + C / 8): 39 A + 2 S + 8 C.
     const float E = 1.2e-7f * (5.0f * asum + 4.0f * s_cmax + 1.0f);
-    const float edd = 1e-14f * (nmax + 2.0f * asum + 2.0f * s_cmax + 2.0f);
+    const float edd = 3.6e-15f * (39.0f * asum + 2.0f * ssum + 8.0f * s_cmax);
     float s_hi[3], s_lo[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -722,14 +733,14 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
 #pragma unroll
         for (int a = 1; a < 3; ++a) {
             float e;
-            ah[a] = two_sum_f((float)(shift[a] + (a == 1 ? y : z)), -s_hi[a], e);
-            al[a] = e - s_lo[a];
+            const float d = two_sum_f((float)(shift[a] + (a == 1 ? y : z)), -s_hi[a], e);
+            ah[a] = two_sum_f(d, e - s_lo[a], al[a]);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             float e;
-            a0h[u] = two_sum_f((float)(shift[0] + x0 + u), -s_hi[0], e);
-            a0l[u] = e - s_lo[0];
+            const float d = two_sum_f((float)(shift[0] + x0 + u), -s_hi[0], e);
+            a0h[u] = two_sum_f(d, e - s_lo[0], a0l[u]);
         }
         float v1[4], v2[4];
         int k1[4];
@@ -764,7 +775,8 @@ k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restric
                 sum = two_sum_f(sum, p2, r1);
                 sum = two_sum_f(sum, f.w, r2);
                 e += lo.w + (r0 + r1 + r2);
-                const float hi = __fadd_rn(sum, e), rest = __fsub_rn(e, __fsub_rn(hi, sum));
+                float rest;
+                const float hi = two_sum_f(sum, e, rest);
                 // the nearest FP32 number of every value within edd
                 const bool sure = v2[u] > v1[u] + 2.0f * E && __fadd_rn(hi, rest + edd) == hi &&
                                   __fadd_rn(hi, rest - edd) == hi;

@@ -369,3 +369,26 @@ def test_neighbour_collection_of_many_boxes(L):
         want = O.predict(ref.grains[g], shape, taps, 7.0, ph, 1.0)
         assert np.max(np.abs(phip[g] - want)) <= 3e-5, g
     assert seen > 16                                 # lists of some length
+
+
+@pytest.mark.parametrize("dims,G,with_weights", [
+    ((8192, 40, 1), 700, False),     # seeds whose FP32 rounding is far above the values' own
+    ((20, 8192, 1), 400, True),
+    ((700, 24, 24), 600, False),
+])
+def test_start_in_wide_domains_against_the_oracle(L, dims, G, with_weights):
+    """As above where a seed's coordinate has few binary places left in FP32: the neighbour that gives the value must
+    still be the right one.  One unit in the last place, for the oracle's own FP64 rounding."""
+    from oracle import lsgg_oracle as O
+    seeds = I.voronoi_seeds(19, G, dims)
+    w = 30.0 * I.u01(19, 6, np.arange(G)) if with_weights else None
+    ref = O.tessellate((dims[2], dims[1], dims[0]), seeds, w)
+    with L.Microstructure(*dims, G, seeds=seeds, weights=w) as ms:
+        boxes, phi = ms.boxes(), ms.phi()
+    for g, r in enumerate(ref.grains):
+        assert bool(boxes[g, 0]) == r.alive
+        if not r.alive:
+            continue
+        assert tuple(boxes[g, 1:4][::-1]) == r.origin and tuple(boxes[g, 4:7][::-1]) == r.dims
+        want = r.phi.astype(np.float32)
+        assert (np.abs(phi[g] - want) <= np.spacing(np.abs(want))).all(), (g, np.max(np.abs(phi[g] - want)))
