@@ -15,6 +15,8 @@
 #include <thread>
 #include <vector>
 
+#include <cuda.h>
+
 #include "bulk_copy.cuh"
 #include "lsgg_internal.cuh"
 #include "../../include/lsgg.h"
@@ -59,6 +61,7 @@ struct lsgg_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    unsigned long long cuda_context = 0; // id of the CUDA context that all of this lives in (0: not known)
     cudaMemPool_t pool = nullptr;        // the device's pool (null: plain allocations)
     std::vector<void*> plain;            // allocations beside it
     Domain dom{};
@@ -149,26 +152,48 @@ int fail_cuda(cudaError_t e) { return trace_cuda(e, 0); }
 // again, and once no context of the device is left it shrinks to kPoolIdle.
 // Allocations and frees are ordered on the context's stream, and memory goes
 // to another stream only after its free has completed.
+// The pool lives in the device's CUDA context and ends with it (a device reset,
+// a released primary context), so it is kept with that context's id: a handle
+// of another id is dropped untouched and a new pool made.
 constexpr size_t kPoolMost = (size_t)512 << 20;
 constexpr unsigned long long kPoolKeep = 4ull << 30, kPoolIdle = 1ull << 30;
 constexpr int kPoolDevices = 64;
 
 struct DevicePool {
     cudaMemPool_t pool = nullptr;
-    bool tried = false;
+    unsigned long long cuda_context = 0;     // where it was made (0: not yet)
     int contexts = 0;
 };
 std::mutex g_pool_mu;
 DevicePool g_pools[kPoolDevices];
 
-// The device's pool with one context more; null (plain allocations) if it
-// has none.
-cudaMemPool_t enter_pool(int device) {
-    if (device < 0 || device >= kPoolDevices) return nullptr;
+// The id of the calling thread's CUDA context, unique in the process' life (0:
+// none, or not to be had).
+unsigned long long cuda_context_id() {
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static const GetId get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<GetId>(f);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// The device's pool in the CUDA context `cuda_context` with one context more;
+// null (plain allocations) if it has none.
+cudaMemPool_t enter_pool(int device, unsigned long long cuda_context) {
+    if (device < 0 || device >= kPoolDevices || !cuda_context) return nullptr;
     std::lock_guard<std::mutex> lk(g_pool_mu);
     DevicePool& d = g_pools[device];
-    if (!d.tried) {
-        d.tried = true;
+    if (d.cuda_context != cuda_context) {
+        d = DevicePool{};
+        d.cuda_context = cuda_context;
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
         props.handleTypes = cudaMemHandleTypeNone;
@@ -191,10 +216,10 @@ cudaMemPool_t enter_pool(int device) {
     return d.pool;
 }
 
-void leave_pool(int device) {
+void leave_pool(int device, unsigned long long cuda_context) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     DevicePool& d = g_pools[device];
-    if (--d.contexts == 0) cudaMemPoolTrimTo(d.pool, kPoolIdle);
+    if (d.cuda_context == cuda_context && --d.contexts == 0) cudaMemPoolTrimTo(d.pool, kPoolIdle);
 }
 
 // From the pool, or plainly where the stream is being captured (a captured
@@ -486,6 +511,11 @@ int lsgg_generate_seeds(uint64_t seed, int32_t n, int32_t nx, int32_t ny, int32_
 int lsgg_destroy(lsgg_ctx* c) {
     if (!c) return LSGG_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    if (c->cuda_context && cuda_context_id() != c->cuda_context) {
+        cudaGetLastError();
+        delete c;                            // its memory, streams and events ended with their CUDA context
+        return LSGG_OK;
+    }
     if (c->stream) cudaStreamSynchronize(c->stream);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->have_ss) {
@@ -503,7 +533,7 @@ int lsgg_destroy(lsgg_ctx* c) {
     for (void* p : c->allocations) device_free(c, p);
     if (c->pool) {
         if (c->stream) cudaStreamSynchronize(c->stream);  // other streams may have the memory now
-        leave_pool(c->device);
+        leave_pool(c->device, c->cuda_context);
     }
     if (c->h_st) cudaFreeHost(c->h_st);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -585,8 +615,9 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) return bail(CUDA_FAIL());
         c->own_stream = true;
     }
-    c->pool = enter_pool(c->device);
     if (cudaMallocHost(&c->h_st, sizeof(StepState)) != cudaSuccess) return bail(LSGG_ERR_OUT_OF_MEMORY);
+    c->cuda_context = cuda_context_id();
+    c->pool = enter_pool(c->device, c->cuda_context);
     std::memset(c->h_st, 0, sizeof(StepState));
     const int G = cfg_in->n_grains;
     c->G = G;

@@ -1,5 +1,8 @@
 """The device memory of contexts that come and go: given back but for a bounded rest, sound for contexts of several
 threads at once, each on its own stream."""
+import os
+import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -64,3 +67,43 @@ def test_memory_is_given_back(L):
     torch.cuda.synchronize()
     assert held > 2 << 30                            # more than the pool keeps without contexts
     assert torch.cuda.mem_get_info()[0] >= free - (1 << 30) - (64 << 20)
+
+
+RESET = """
+import ctypes, numpy as np
+from paper_1701_06658_gb300 import inputs as I, lsgg as L
+L.lib()
+rt = ctypes.CDLL("libcudart.so.13")
+
+def run(keep=False):
+    ms = L.Microstructure(40, 36, 44, 12, seeds=I.voronoi_seeds(3, 12, (40, 36, 44)))
+    ms.step(4, 1.0)
+    ms.sync()
+    out = ms.boxes(), L.get_phi(ms.ctx), ms.grain_volumes()
+    if keep:
+        return ms, out
+    ms.close()
+    return out
+
+want = run()
+old, _ = run(keep=True)
+for k in range(2):
+    assert rt.cudaDeviceReset() == 0
+    ms, got = run(keep=True)
+    assert all(np.array_equal(a, b) for a, b in zip(want, got))
+    old.close()                                      # of the CUDA context before: nothing of the new one goes with it
+    assert all(np.array_equal(a, b) for a, b in zip(want, run()))
+    assert np.array_equal(want[1], L.get_phi(ms.ctx))
+    old = ms
+print("same after the reset")
+"""
+
+
+def test_contexts_after_a_device_reset():
+    """The process ends its own CUDA context (cudaDeviceReset) with a microstructure in it and makes new ones."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=root, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "same after the reset" in r.stdout, r.stderr[-2000:]
