@@ -226,21 +226,24 @@ void leave_pool(int device, unsigned long long cuda_context) {
 // allocation would belong to the graph).
 cudaError_t device_malloc(lsgg_ctx* c, void** q, size_t bytes) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool pooled = c->pool && bytes <= kPoolMost;
-    if (pooled && (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)) {
+    const bool capturing =
+        c->pool && (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone);
+    if (capturing) cudaGetLastError();
+    // all that the pool holds unused back to the device
+    auto give_back = [&] {
         cudaGetLastError();
-    } else if (pooled) {
+        if (!capturing) cudaStreamSynchronize(c->stream);  // frees of this stream complete: pending ones stay
+        cudaMemPoolTrimTo(c->pool, 0);
+    };
+    if (c->pool && bytes <= kPoolMost && !capturing) {
         cudaError_t e = cudaMallocFromPoolAsync(q, bytes, c->pool, c->stream);
         if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-        cudaStreamSynchronize(c->stream);                 // frees of this stream complete
-        cudaMemPoolTrimTo(c->pool, 0);
+        give_back();
         return cudaMallocFromPoolAsync(q, bytes, c->pool, c->stream);
     }
     cudaError_t e = cudaMalloc(q, bytes);
     if (e == cudaErrorMemoryAllocation && c->pool) {
-        cudaGetLastError();
-        cudaMemPoolTrimTo(c->pool, 0);
+        give_back();
         e = cudaMalloc(q, bytes);
     }
     if (e == cudaSuccess && c->pool) c->plain.push_back(*q);

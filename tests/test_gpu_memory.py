@@ -69,6 +69,35 @@ def test_memory_is_given_back(L):
     assert torch.cuda.mem_get_info()[0] >= free - (1 << 30) - (64 << 20)
 
 
+def test_growth_from_the_pool_to_plain_allocations(L):
+    """An arena grows past the size up to which buffers come from the pool, with room for the new ones only if the
+    old ones, just freed into the pool, are given back: the room left holds three of the four new buffers."""
+    import torch
+    dims, G = (96, 96, 96), 60
+    e = 4e-2 * I.u01(5, 7, np.arange(G))
+    old_cap, new_cap = 110 << 20, 150 << 20          # elements of four bytes: 440 and 600 MiB a buffer
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(5, G, dims), energy=e, physics=L.PHYSICS_MAGNETIC) as a, \
+            L.Microstructure(*dims, G, seeds=I.voronoi_seeds(5, G, dims), energy=e, physics=L.PHYSICS_MAGNETIC) as b:
+        a.step(4, 1.0)
+        a.sync()
+        L.debug_set_capacity(b.ctx, old_cap)
+        b.step(2, 1.0)
+        b.sync()
+        torch.cuda.synchronize()
+        room = 3 * 4 * new_cap + (256 << 20)
+        ballast = torch.empty(max(0, torch.cuda.mem_get_info()[0] - room), dtype=torch.uint8, device="cuda")
+        try:
+            L.debug_set_capacity(b.ctx, new_cap)     # raises when it runs out
+        finally:
+            del ballast
+            torch.cuda.empty_cache()
+        b.step(2, 1.0)
+        b.sync()
+        assert b.stats().arena_capacity == new_cap
+        assert np.array_equal(a.boxes(), b.boxes())
+        assert np.array_equal(L.get_phi(a.ctx), L.get_phi(b.ctx))
+
+
 RESET = """
 import ctypes, numpy as np
 from paper_1701_06658_gb300 import inputs as I, lsgg as L
