@@ -339,10 +339,12 @@ int lsgg_profile(lsgg_ctx* ctx, int32_t enable);
 
 /* Tile autotuner of the batched path.  On the pass path (3D boxes) it runs
  * four trials of steps_per_trial profiled steps each -- every persistent grid
- * at the CTAs per SM that fit, every grid at half of that, and slab items of
- * 4 and 16 planes for the re-initialisation's plane pass instead of 8 -- and
- * keeps per tier and pass the faster grid and the slab with the least plane
- * pass time (read back with lsgg_pass_tuning); chosen (optional, 2 x 8
+ * at the CTAs per SM that fit, every grid at half of that, both with the
+ * context's own depth of the slab items, and the other two of the depths 4, 8
+ * and 16 planes -- and keeps per tier and pass the faster grid, and the depth
+ * with the least time of the plane passes that walk slabs (read back with
+ * lsgg_pass_tuning).  With few box planes every depth is halved as the
+ * context's own is, so that the items still go round; chosen (optional, 2 x 8
  * int32) is then all -1.  Otherwise, for every box-size class served by the
  * register-ring kernels, it runs steps_per_trial real steps with each tile
  * variant (cells per thread, threads per CTA), times each class's kernels
@@ -357,8 +359,9 @@ int lsgg_autotune(lsgg_ctx* ctx, int32_t steps_per_trial, double dt, int32_t* ch
 /* The pass path's current tuning: ctas_per_sm (optional, 4 * LSGG_PASS_TIERS
  * int32) the CTAs per SM of the persistent grids of p_conv_xy, p_conv_z,
  * p_redist_xy and p_redist_z of each tier, slab (optional) the planes per slab
- * item of the plane passes (before a tuning 16, 8, 4 or 2 by the number of
- * box planes); -1 off the pass path. */
+ * item of the plane passes: before a tuning the depth in use, 16, 8, 4 or 2 by
+ * the number of box planes; after one the depth it chose, 4, 8 or 16, which
+ * few box planes make shallower in use.  -1 off the pass path. */
 int lsgg_pass_tuning(lsgg_ctx* ctx, int32_t* ctas_per_sm, int32_t* slab);
 int lsgg_kernel_times(lsgg_ctx* ctx, double* out_ms, int64_t* out_count);
 
@@ -573,6 +576,10 @@ int lsgg_closest_gb_map(const lsgg_box* boxes_dev, int32_t n_boxes, const float*
  * elements (at least what the current state needs), so that a later box update
  * overflows and exercises the growth path of lsgg_sync.  Synchronises. */
 int lsgg_debug_set_capacity(lsgg_ctx* ctx, int64_t capacity);
+
+/* Test hook: the planes per slab item in use (lsgg_pass_tuning's slab, halved
+ * while the box planes are too few for it); -1 off the pass path. */
+int lsgg_debug_slab_depth(lsgg_ctx* ctx, int32_t* depth);
 
 /* Test hook of the bounded device waits: one CTA initialises an mbarrier that
  * nothing will complete and waits on it for at most `iterations` polls, the

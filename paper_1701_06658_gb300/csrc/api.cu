@@ -101,6 +101,7 @@ struct lsgg_ctx {
     StepStreams ss{};
     bool have_ss = false;
     bool separate_z = false;         // pass path with an ID-field: Z has its own arena
+    int tuned_slab = 0;              // the autotuner's slab depth (0: not tuned)
     // plain (per-grain) comparator buffers
     float *p_t1 = nullptr, *p_t2 = nullptr, *p_C = nullptr, *p_G = nullptr, *p_H = nullptr;
     long long p_cap = 0;
@@ -444,6 +445,17 @@ int relayout(lsgg_ctx* c) {
         return LSGG_OK;
     }
     return LSGG_ERR_OUT_OF_MEMORY;
+}
+
+// The slab depth (B.slab) for boxes of `planes` planes in all: the tuned one,
+// or kDeepSlab or kSlab by their number; less while that leaves too few slab
+// items to go round (a shorter slab loads and classifies more planes twice, a
+// longer one leaves SMs idle).
+void set_slab(lsgg_ctx* c, long long planes) {
+    int slab = c->tuned_slab;
+    if (!slab) slab = planes >= (long long)kDeepItemsPerSm * c->B.n_sm * kDeepSlab ? kDeepSlab : kSlab;
+    while (slab > kMinSlab && planes < (long long)kSlabItemsPerSm * c->B.n_sm * slab) slab /= 2;
+    c->B.slab = slab;
 }
 
 int enqueue_steps(lsgg_ctx* c, long long n, double dt, const DebugOut* dbg);
@@ -872,12 +884,9 @@ static int create_impl(const lsgg_config* cfg_in, void* stream, lsgg_ctx** out) 
         if ((r = dalloc(c, &c->B.scratch, (size_t)std::max(total, 32LL))) != LSGG_OK) return bail(r);
     }
     if (c->B.use_passes) {
-        // slab items enough to go round: a shorter slab loads and classifies
-        // more planes twice, a longer one leaves SMs idle
         long long planes = 0;
         for (const Box& b : hb) planes += b.nz;
-        if (planes >= (long long)kDeepItemsPerSm * c->B.n_sm * kDeepSlab) c->B.slab = kDeepSlab;
-        while (c->B.slab > kMinSlab && planes < (long long)kSlabItemsPerSm * c->B.n_sm * c->B.slab) c->B.slab /= 2;
+        set_slab(c, planes);
     }
     if ((r = relayout(c)) != LSGG_OK) return bail(r);
     c->phys.kind = cfg_in->physics;
@@ -1218,30 +1227,41 @@ int lsgg_get_stats(lsgg_ctx* c, lsgg_stats* out) {
 
 // The pass path's tunables: per tier and pass the CTAs per SM of its
 // persistent grid (pgrid index 0 conv_xy, 1 / 2 conv_z ideal / physics, 3
-// redist_xy, 4 redist_z) and the slab depth of p_redist_xy.  Re-lays the work
-// items out for the slab; the step graph is captured anew.
+// redist_xy, 4 redist_z) and the slab depth of the plane passes, which few
+// planes still make shallower (set_slab).  Re-lays the work items out for the
+// slab; the step graph is captured anew.
 static int apply_pass_tuning(lsgg_ctx* c, const int (&ctas)[kTiers][5], int slab) {
     for (int t = 0; t < kTiers; ++t)
         for (int k = 0; k < 5; ++k) c->B.pgrid[t][k] = c->B.n_sm * std::max(1, std::min(ctas[t][k], c->B.pocc[t][k]));
-    c->B.slab = slab;
+    int r = read_state(c);
+    if (r != LSGG_OK) return r;
+    long long planes = 0;
+    for (int t = 0; t < kTiers; ++t) planes += c->h_st->n_planes[t];
+    c->tuned_slab = slab;
+    set_slab(c, planes);
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
     return relayout(c);
 }
 
 // Autotuner of the pass path: trials of steps_per_trial profiled steps each
-// with (a) every grid at its resident maximum and the default slab, (b) every
-// grid at half of it, (c, d) slabs of half and twice the default; per tier and
-// pass the faster grid of (a, b), and the slab with the least
-// re-initialisation plane-pass time over the tiers.  All settings give bit-identical steps.
+// with (a) every grid at its resident maximum and the context's own slab depth,
+// (b) every grid at half of it, (c, d) the other two of the depths 4, 8 and 16;
+// per tier and pass the faster grid of (a, b), and the depth with the least time
+// of the two passes that walk slabs (p_conv_xy, p_redist_xy) over the tiers.  A
+// depth that few planes make the same as the own one (set_slab) is not preferred
+// to it.  All settings give bit-identical steps.
 static int autotune_passes(lsgg_ctx* c, int32_t steps_per_trial, double dt) {
     int full[kTiers][5], half[kTiers][5];
     for (int t = 0; t < kTiers; ++t)
         for (int k = 0; k < 5; ++k) { full[t][k] = c->B.pocc[t][k]; half[t][k] = std::max(1, c->B.pocc[t][k] / 2); }
-    const int slabs[4] = {kSlab, kSlab, kSlab / 2, 2 * kSlab};
+    const int own = c->tuned_slab ? c->tuned_slab : std::max(c->B.slab, kSlab);
+    const int slabs[4] = {own, own, own == kSlab / 2 ? kSlab : kSlab / 2, own == 2 * kSlab ? kSlab : 2 * kSlab};
+    int depth[4];
     double ms[4][kTiers * 4 + 2] = {};
     c->profiling = true;
     for (int trial = 0; trial < 4; ++trial) {
         int r = apply_pass_tuning(c, trial == 1 ? half : full, slabs[trial]);
+        depth[trial] = c->B.slab;
         if (r == LSGG_OK) r = lsgg_step(c, steps_per_trial, dt);
         if (r == LSGG_OK) r = lsgg_pass_times(c, ms[trial], nullptr);
         if (r != LSGG_OK) { c->profiling = false; return r; }
@@ -1256,12 +1276,12 @@ static int autotune_passes(lsgg_ctx* c, int32_t steps_per_trial, double dt) {
                 const int k = pk[q][j];
                 best[t][k] = ms[1][t * 4 + q] < ms[0][t * 4 + q] ? half[t][k] : full[t][k];
             }
-    int slab = kSlab;
+    int slab = own;
     double slab_ms = 0.0;
     for (int trial : {0, 2, 3}) {
         double tot = 0.0;
-        for (int t = 0; t < kTiers; ++t) tot += ms[trial][t * 4 + 2];
-        if (trial == 0 || tot < slab_ms) { slab_ms = tot; slab = slabs[trial]; }
+        for (int t = 0; t < kTiers; ++t) tot += ms[trial][t * 4] + ms[trial][t * 4 + 2];
+        if (trial == 0 || (tot < slab_ms && depth[trial] != depth[0])) { slab_ms = tot; slab = slabs[trial]; }
     }
     return apply_pass_tuning(c, best, slab);
 }
@@ -1273,7 +1293,7 @@ int lsgg_pass_tuning(lsgg_ctx* c, int32_t* ctas_per_sm, int32_t* slab) {
             const int k4[4] = {0, c->phys.kind != LSGG_PHYSICS_IDEAL ? 2 : 1, 3, 4};
             for (int q = 0; q < 4; ++q) ctas_per_sm[t * 4 + q] = c->B.use_passes ? c->B.pgrid[t][k4[q]] / c->B.n_sm : -1;
         }
-    if (slab) *slab = c->B.use_passes ? c->B.slab : -1;
+    if (slab) *slab = !c->B.use_passes ? -1 : c->tuned_slab ? c->tuned_slab : c->B.slab;
     return LSGG_OK;
 }
 
@@ -1454,6 +1474,12 @@ int lsgg_debug_set_capacity(lsgg_ctx* c, int64_t capacity) {
     if ((r = ensure_chunk_cap(c)) != LSGG_OK) return r;
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
     return relayout(c);
+}
+
+int lsgg_debug_slab_depth(lsgg_ctx* c, int32_t* depth) {
+    if (!c || !depth) return LSGG_ERR_INVALID_ARG;
+    *depth = c->B.use_passes ? c->B.slab : -1;
+    return LSGG_OK;
 }
 
 int lsgg_debug_set_wait_limit(lsgg_ctx* c, int32_t polls) {
@@ -1782,6 +1808,9 @@ int lsgg_coarsen(lsgg_ctx* c, int32_t nx, int32_t ny, int32_t nz) {
     if ((r = dalloc(c, &d_fine, (size_t)c->G)) != LSGG_OK) return r;
     r = to_device(c, d_fine, hp.data(), (size_t)c->G * sizeof(Box)) == cudaSuccess ? LSGG_OK
                                                                                                      : LSGG_ERR_CUDA;
+    long long planes = 0;
+    for (const Box& b : hc) planes += b.nz;
+    set_slab(c, planes);
     if (r == LSGG_OK) r = relayout(c);
     // projection into Z, then the re-initialisation and box update of a step
     const float* x = nullptr;

@@ -38,8 +38,8 @@ constexpr int kFewBoxes = 2048;         // up to this many boxes, kernels of a C
 constexpr int kPassChunk = 256;         // columns per column item of the pass path
 constexpr int kSlab = 8;                // planes per slab item of the pass path (default; autotuned)
 constexpr int kMinSlab = 2;             // the smallest slab (sizes the slab item list)
-// The slab is halved while the initial boxes give fewer slab items per SM than
-// this.  Measured on GB300, a step with the slab so found and with 8 planes:
+// The slab (tuned or not) is halved while the boxes at creation, tuning or
+// coarsening give fewer slab items per SM than this.  Measured on GB300, a step with the slab so found and with 8 planes:
 // 32^3 / 20 grains 0.093 and 0.112 ms, 64^3 / 50 0.089 and 0.108.  With the
 // line at 8 or 16 149 x 97 x 61 / 263 would gain too (0.164 against 0.175 ms),
 // but a served mix of 24 requests, whose groups fill the GPU, takes 164 or

@@ -130,6 +130,7 @@ _SIGS = {
     "lsgg_grain_neighbours": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.c_int32]),
     "lsgg_keep_field": (C.c_int, [C.c_void_p, C.c_int32]),
     "lsgg_autotune": (C.c_int, [C.c_void_p, C.c_int32, C.c_double, C.POINTER(C.c_int32)]),
+    "lsgg_debug_slab_depth": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32)]),
     "lsgg_pass_tuning": (C.c_int, [C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "lsgg_debug_set_capacity": (C.c_int, [C.c_void_p, C.c_int64]),
     "lsgg_debug_wait_timeout": (C.c_int, [C.c_int32, C.c_int32, C.POINTER(C.c_int32)]),
@@ -295,6 +296,13 @@ def autotune(ctx, steps_per_trial: int = 2, dt: float = 1.0) -> dict:
     chosen = np.full(16, -1, np.int32)
     _check("autotune", lib().lsgg_autotune(ctx, steps_per_trial, float(dt), _ptr(chosen, C.c_int32)))
     return {"k_predict": chosen[0:5].tolist(), "k_correct": chosen[5:10].tolist()}
+
+
+def debug_slab_depth(ctx) -> int:
+    """Test hook: planes per slab item in use."""
+    depth = C.c_int32()
+    _check("debug_slab_depth", lib().lsgg_debug_slab_depth(ctx, C.byref(depth)))
+    return depth.value
 
 
 def pass_tuning(ctx) -> dict:

@@ -392,3 +392,21 @@ def test_start_in_wide_domains_against_the_oracle(L, dims, G, with_weights):
         assert tuple(boxes[g, 1:4][::-1]) == r.origin and tuple(boxes[g, 4:7][::-1]) == r.dims
         want = r.phi.astype(np.float32)
         assert (np.abs(phi[g] - want) <= np.spacing(np.abs(want))).all(), (g, np.max(np.abs(phi[g] - want)))
+
+
+@pytest.mark.parametrize("dims,G,own", [((32, 32, 32), 20, 2), ((64, 64, 64), 50, 2), ((64, 64, 64), 95, 4)])
+def test_tuning_keeps_the_depth_of_few_planes(L, dims, G, own):
+    """A small microstructure's slab items hold few planes; a tuning leaves it at that depth, whatever depth it chose
+    for more planes."""
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(1, G, dims)) as ms:
+        assert L.debug_slab_depth(ms.ctx) == own
+        L.autotune(ms.ctx, 2, 1.0)
+        assert L.debug_slab_depth(ms.ctx) == own
+
+
+def test_coarsening_takes_the_depth_of_the_coarse_boxes(L):
+    dims, G = (64, 64, 64), 95
+    with L.Microstructure(*dims, G, seeds=I.voronoi_seeds(1, G, dims)) as ms:
+        assert L.debug_slab_depth(ms.ctx) == 4
+        L.coarsen(ms.ctx, 32, 32, 32)
+        assert L.debug_slab_depth(ms.ctx) == 2
