@@ -19,7 +19,14 @@
  *     lsgg_status_string() names it.  No function throws or aborts.
  *   - host pointers are caller-owned; the library copies what it needs and
  *     keeps no host pointer after the call returns.
- *   - a context owns all of its device memory; lsgg_destroy frees it.
+ *   - a context owns all of its device memory; lsgg_destroy frees it.  Buffers
+ *     of up to 512 MiB come from a memory pool that the library keeps per device
+ *     for its contexts: of freed memory it holds at most 4 GiB back for reuse
+ *     while a context of the device lives and at most 1 GiB after the last one
+ *     is destroyed, until the CUDA context ends.  An allocation of the library
+ *     that finds no room gives all of that back first; other allocators of the
+ *     process do not see it as free.  It is in no context's device_bytes and in
+ *     no server's budget.
  *   - a context is not thread-safe; distinct contexts are independent.
  *   - every device computation runs in the library's CUDA kernels; there is
  *     no CPU fallback.  Without a usable CUDA device, calls that compute
@@ -194,8 +201,8 @@ int lsgg_group_destroy(lsgg_group* g);
  * The paper does not define a grain's volume; this is a smooth cell count:
  * the zero level of phi_i smeared over one cell, so that it moves
  * continuously with the interface (the volumes the grain-size analysis of
- * Sec. 5 takes its equivalent radii from).  Computed from exact fixed-point
- * partial sums merged with FP64 compensated sums in a fixed order
+ * Sec. 5 takes its equivalent radii from).  Computed as one exact fixed-point
+ * sum (units of 2^-28, the same in any order), rounded once to FP64
  * (deterministic); index = grain id, 0 for extinct grains.  out: host array
  * of cap >= n_grains doubles; *n_out = n_grains.  Synchronises. */
 int lsgg_grain_volumes(lsgg_ctx* ctx, double* out, int64_t cap, int64_t* n_out);
@@ -290,7 +297,9 @@ int lsgg_voxel_owner(lsgg_ctx* ctx, int32_t* out, int64_t n_cells);
 int lsgg_grain_volumes_device(lsgg_ctx* ctx, double* out_dev, int64_t cap, int32_t* status_dev, void* stream);
 int lsgg_voxel_owner_device(lsgg_ctx* ctx, int32_t* out_dev, int64_t n_cells, int32_t* status_dev, void* stream);
 
-/* Free all device memory of the context (after finishing its work). */
+/* Free all device memory of the context (after finishing its work); the
+ * device's pool may keep up to 1 GiB of freed memory, 4 GiB while other
+ * contexts live (see the conventions above). */
 int lsgg_destroy(lsgg_ctx* ctx);
 
 const char* lsgg_status_string(int status);
