@@ -1284,7 +1284,9 @@ cudaError_t launch_step(const StepBuffers& B, const Taps& taps, const PhysicsDev
 // update that counts no step.  With id_field, the field pass then runs on the
 // re-initialised state (copied to Y as its phi_p) before the box update, so
 // that the ID-field the next step's correction reads exists in this layout.
-// Used by the grid coarsening.
+// Used by the grid coarsening and the label start; every tier is launched, since
+// a coarsening's layout takes a box's tier from the larger of its fine and its
+// coarse sides.
 cudaError_t launch_reinit(const StepBuffers& B, const Taps& taps, const PhysicsDev& phys, bool id_field,
                           cudaStream_t s) {
     if (!B.use_passes) return cudaErrorInvalidValue;
