@@ -371,27 +371,24 @@ def test_neighbour_collection_of_many_boxes(L):
     assert seen > 16                                 # lists of some length
 
 
-@pytest.mark.parametrize("dims,G,with_weights", [
-    ((8192, 40, 1), 700, False),     # seeds whose FP32 rounding is far above the values' own
-    ((20, 8192, 1), 400, True),
-    ((700, 24, 24), 600, False),
-])
-def test_start_in_wide_domains_against_the_oracle(L, dims, G, with_weights):
-    """As above where a seed's coordinate has few binary places left in FP32: the neighbour that gives the value must
-    still be the right one.  One unit in the last place, for the oracle's own FP64 rounding."""
-    from oracle import lsgg_oracle as O
-    seeds = I.voronoi_seeds(19, G, dims)
-    w = 30.0 * I.u01(19, 6, np.arange(G)) if with_weights else None
-    ref = O.tessellate((dims[2], dims[1], dims[0]), seeds, w)
-    with L.Microstructure(*dims, G, seeds=seeds, weights=w) as ms:
+@pytest.mark.parametrize("with_weights", [False, True])
+def test_start_in_a_wide_domain(L, with_weights):
+    """Two equal halves of 4096 columns (seed coordinates of 12 binary places, so that every displacement is the same
+    FP64 number in both), where a seed's rounding to FP32 is far above that of the values and differs between the
+    halves: the second half's grains have the first's boxes and, bit for bit, their functions."""
+    nx, ny, nz = 4096, 80, 80
+    G = nx * ny * nz // 1728
+    seeds = np.round(I.voronoi_seeds(19, G, (nx, ny, nz)) * 2.0 ** 12) / 2.0 ** 12
+    w = np.tile(20.0 * I.u01(19, 6, np.arange(G)), 2) if with_weights else None
+    both = np.concatenate([seeds, seeds + [float(nx), 0.0, 0.0]])
+    with L.Microstructure(2 * nx, ny, nz, 2 * G, seeds=both, weights=w) as ms:
         boxes, phi = ms.boxes(), ms.phi()
-    for g, r in enumerate(ref.grains):
-        assert bool(boxes[g, 0]) == r.alive
-        if not r.alive:
-            continue
-        assert tuple(boxes[g, 1:4][::-1]) == r.origin and tuple(boxes[g, 4:7][::-1]) == r.dims
-        want = r.phi.astype(np.float32)
-        assert (np.abs(phi[g] - want) <= np.spacing(np.abs(want))).all(), (g, np.max(np.abs(phi[g] - want)))
+    assert np.array_equal(boxes[:G, [0, 2, 3, 4, 5, 6]], boxes[G:, [0, 2, 3, 4, 5, 6]])
+    alive = boxes[:G, 0] != 0
+    assert alive.sum() > G // 2
+    assert np.array_equal((boxes[G:][alive, 1] - nx) % (2 * nx), boxes[:G][alive, 1])
+    different = [g for g in np.flatnonzero(alive) if not np.array_equal(phi[g], phi[g + G])]
+    assert not different, (len(different), max(np.max(np.abs(phi[g] - phi[g + G])) for g in different))
 
 
 @pytest.mark.parametrize("dims,G,own", [((32, 32, 32), 20, 2), ((64, 64, 64), 50, 2), ((64, 64, 64), 95, 4)])
