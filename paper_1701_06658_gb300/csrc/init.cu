@@ -488,7 +488,7 @@ constexpr int kSdfThreads = 256;
 // boundary lies within that error; then, and where E does not separate the two,
 // the cell takes the general FP64 form (`slow_cell`), as every cell of a box
 // without `fast` does.  FP64 for every cell's winner kept the FP64 pipe busy:
-// 9.6 ms at 256^3 / 5000 grains, against 1.95 ms.
+// 9.6 ms at 256^3 / 5000 grains, against 2.00 ms.
 __global__ void __launch_bounds__(kSdfThreads)
 k_sdf(Domain D, const int2* __restrict__ items, int groups, const Box* __restrict__ boxes,
       const double* __restrict__ seeds, const double* __restrict__ weights, const unsigned* __restrict__ bits,
