@@ -183,7 +183,11 @@ unsigned long long cuda_context_id() {
         return reinterpret_cast<GetId>(f);
     }();
     unsigned long long id = 0;
-    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+    if (!get) return 0;
+    if (get(nullptr, &id) == CUDA_SUCCESS) return id;
+    size_t free_b = 0, total_b = 0;              // a thread without one yet: the runtime's first call that needs it binds it
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) cudaGetLastError();
+    return get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
 }
 
 // The device's pool in the CUDA context `cuda_context` with one context more;
@@ -526,8 +530,8 @@ int lsgg_generate_seeds(uint64_t seed, int32_t n, int32_t nx, int32_t ny, int32_
 int lsgg_destroy(lsgg_ctx* c) {
     if (!c) return LSGG_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
-    if (c->cuda_context && cuda_context_id() != c->cuda_context) {
-        cudaGetLastError();
+    const unsigned long long now = c->cuda_context ? cuda_context_id() : 0;
+    if (now && now != c->cuda_context) {
         delete c;                            // its memory, streams and events ended with their CUDA context
         return LSGG_OK;
     }

@@ -69,6 +69,27 @@ def test_memory_is_given_back(L):
     assert torch.cuda.mem_get_info()[0] >= free - (1 << 30) - (64 << 20)
 
 
+def test_a_thread_new_to_cuda_destroys_contexts(L):
+    """Contexts made by this thread and destroyed by one that has called nothing of CUDA: their memory is back."""
+    import torch
+    _run(L, 1)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    n, G = 128, 600
+    mss = [L.Microstructure(n, n, n, G, seeds=I.voronoi_seeds(k, G, (n, n, n))) for k in range(6)]
+    assert sum(ms.stats().device_bytes for ms in mss) > 2 << 30
+
+    def close():
+        for ms in mss:
+            ms.close()
+
+    t = threading.Thread(target=close)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] >= free - (1 << 30) - (64 << 20)
+
+
 def test_growth_from_the_pool_to_plain_allocations(L):
     """An arena grows past the size up to which buffers come from the pool, with room for the new ones only if the
     old ones, just freed into the pool, are given back: the room left holds three of the four new buffers."""
